@@ -50,15 +50,6 @@ __device__ __forceinline__ int poff(int c) { return (c * (c + 3)) >> 1; }
 // walls: nothing swaps with them and they do not move.
 constexpr uint8_t SEL_WALL = 3;
 
-// ---------------------------------------------------------------------------
-// 2|2 swap by 16 lanes.  The sequential part (Sylvester elimination with
-// complete pivoting, the two reflectors) is computed redundantly by every
-// lane -- an FP64 instruction costs the same for 1 or 16 lanes -- and the
-// 4x4 products (Qs, Qs^T D Qs, the strong test) are lane-parallel: lane l of
-// the half-warp owns entry (r, c) = (l & 3, l >> 2).  No re-standardization
-// (done at the end of the window).  Returns false if the fast path cannot
-// decide; the caller then runs the full transform.
-// ---------------------------------------------------------------------------
 __device__ __forceinline__ double sel4(int i, double a0, double a1, double a2, double a3) {
     return i == 0 ? a0 : (i == 1 ? a1 : (i == 2 ? a2 : a3));
 }
@@ -152,66 +143,223 @@ __device__ __forceinline__ bool sylv22_regs(const double* D, double* X) {
     return true;
 }
 
-// Returns true (and this lane's Z and Dn entries) if the fast path decided
-// the swap and accepted it; *fallback is set when the full transform must run.
-__device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, int ja, int l,
-                                                unsigned hmask, int hbase, bool strong,
-                                                double* zrc, double* dnrc, bool* fallback) {
-    const int r = l & 3, c = l >> 2;
+// ---------------------------------------------------------------------------
+// Building blocks of the swap transforms.  What bounds a transform: on this
+// part a warp's FP64 instruction holds its sub-partition's pipe for 64 cycles
+// and its result is 64 cycles away, whatever the number of active lanes, while
+// FP32 and integer instructions cost a cycle or two.  So the transforms keep
+// the number of FP64 instructions down: first approximations come from the
+// special function unit or from FP32, and FP64 only corrects them.  Measured
+// against transforms in FP64 throughout, with 3x3 and 4x4 products: a window
+// task of w = 128, m = 64 took 1.90 ms and takes 1.48 ms (median in the
+// n = 4000 schedule), one of w = 32, m = 16 took 268 us and takes 193 us; the
+// rounding errors of whole reorderings (orthogonality, residual, swaps sent to
+// the double-double retry) are a little smaller than they were.
+// ---------------------------------------------------------------------------
+// Seeds with about 20 correct bits (PTX rcp/rsqrt.approx.ftz.f64).
+__device__ __forceinline__ double rcp_seed(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+__device__ __forceinline__ double rsqrt_seed(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+// x times 2^-1 for a normal x above the smallest binade.
+__device__ __forceinline__ double half_of(double x) {
+    return __longlong_as_double(__double_as_longlong(x) - (1LL << 52));
+}
+// 1/x for normal x: one third-order step, y (1 + e + e^2) with e = 1 - x y
+// (the geometric series of 1 / (1 - e)).
+__device__ __forceinline__ double rcp64(double x) {
+    const double y = rcp_seed(x), e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// sqrt(x) for normal x: one step of Goldschmidt's iteration on (sqrt, 1/(2
+// sqrt)) and a final residual correction (Markstein 2004).
+__device__ __forceinline__ double sqrt64(double x) {
+    const double y = rsqrt_seed(x);
+    double g = x * y, h = half_of(y);
+    const double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    return fma(fma(-g, g, x), h, g);
+}
+// Reflector I - f w w^T with w = (w0, a1, 1) that maps a = (a0, a1, 1) onto
+// -sign(a0) |a| e_0: w0 = a0 + sign(a0) |a|, f = 2 / |w|^2 (taken from the
+// rounded w, so that only f's own rounding touches the orthogonality).  The
+// last component of w stays 1, so that applying it takes six FP64
+// instructions (a 3x3 product takes nine).
+__device__ __forceinline__ void refl3(double a0, double a1, double* w0, double* f) {
+    const double n1 = fma(a1, a1, 1.0);
+    const double d = fabs(a0) + sqrt64(fma(a0, a0, n1));
+    *w0 = a0 >= 0.0 ? d : -d;
+    *f = rcp64(half_of(fma(d, d, n1)));
+}
+__device__ __forceinline__ void apply_refl3(double w0, double w1, double f, double* x0, double* x1,
+                                            double* x2) {
+    const double s = fma(w0, *x0, fma(w1, *x1, *x2)) * f;
+    *x0 = fma(-s, w0, *x0);
+    *x1 = fma(-s, w1, *x1);
+    *x2 -= s;
+}
+// x 2^(127 - eoff) as a float by truncation, and a float as a double, both on
+// the integer pipe (0 below the normal range, infinity above it).
+__device__ __forceinline__ float to_f32(double x, int eoff) {
+    const unsigned hi = __double2hiint(x), lo = __double2loint(x);
+    const int fld = (int)((hi >> 20) & 0x7ff), e = fld - eoff;
+    const unsigned b = e <= 0 || fld == 0 ? 0u
+                     : e >= 255 ? 0x7f800000u
+                                : ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    return __uint_as_float((hi & 0x80000000u) | b);
+}
+__device__ __forceinline__ double from_f32(float x) {
+    const unsigned b = __float_as_uint(x), e = (b >> 23) & 255u;
+    if (e == 0) return 0.0;
+    return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)),
+                            (int)(b << 29));
+}
+
+// The elimination kept for the swaps whose FP32-seeded solution does not
+// converge (out of line: it is rare, and the step loop must fit the
+// instruction caches).
+static __device__ __noinline__ bool sylv22_full(const double* __restrict__ Sp, int ja, double* X) {
     double D[16];
 #pragma unroll
     for (int cc = 0; cc < 4; ++cc)
 #pragma unroll
         for (int rr = 0; rr < 4; ++rr)
             D[cc * 4 + rr] = (rr <= cc + 1) ? Sp[poff(ja + cc) + ja + rr] : 0.0;
-    *fallback = false;
-    unsigned long long mx = 0;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) mx = abs_bits(D[i]) > mx ? abs_bits(D[i]) : mx;
+    return sylv22_regs(D, X);
+}
+
+// 2|2 swap by 16 lanes: lane l of the half-warp owns entry (r, c) =
+// (l & 3, l >> 2) of the 4x4 matrices.  No re-standardization (done at the end
+// of the window).  Returns false if the full transform must run; otherwise
+// *dnrc is this lane's entry of the new block and z holds the two reflectors,
+// (w0, w1, f) on rows 0..2 and (u0, u1, f') on rows 1..3.
+//
+// The Sylvester equation A X - X B = C (T11 = A, T22 = B, T12 = C, both
+// diagonal blocks shifted by B's first diagonal entry, which cancels) is
+// solved in closed form: M X = A C - C adj(B) with M = A^2 - tr(B) A + det(B) I
+// (Cayley-Hamilton on B), evaluated in FP32, then refined with FP64 residuals
+// until a correction c has |c| <= 2^-36 |X|: corrections shrink by the same
+// factor each time, and two of them that reach 2^-36 leave an error below
+// 2^-53.  Two corrections are the rule; a solution that does not get there in
+// six goes to the elimination with complete pivoting.
+// FP64 instructions: 3 + 5 per correction, 30 for the reflectors, 22 for the
+// products and tests; the elimination in FP64, two square roots and five
+// divisions took about 200.
+__device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, int ja, int l,
+                                                unsigned hmask, int hbase, bool strong,
+                                                double* z, double* dnrc) {
+    const int r = l & 3, c = l >> 2;
+    const double* c0 = Sp + poff(ja) + ja;
+    const double* c1 = Sp + poff(ja + 1) + ja;
+    const double* c2 = Sp + poff(ja + 2) + ja;
+    const double* c3 = Sp + poff(ja + 3) + ja;
+    const double b00 = c2[2];
+    const double a00 = c0[0] - b00, a10 = c0[1], a01 = c1[0], a11 = c1[1] - b00;
+    const double b10 = c2[3], b01 = c3[2], b11 = c3[3] - b00;
+    // this lane's column of D and the largest entry of D
+    const double* cc = Sp + poff(ja + c) + ja;
+    const double dc0 = cc[0], dc1 = cc[1], dc2 = c >= 1 ? cc[2] : 0.0, dc3 = c >= 2 ? cc[3] : 0.0;
+    unsigned long long mx = abs_bits(dc0), t1 = abs_bits(dc1), t2 = abs_bits(dc2), t3 = abs_bits(dc3);
+    mx = t1 > mx ? t1 : mx;
+    t2 = t3 > t2 ? t3 : t2;
+    mx = t2 > mx ? t2 : mx;
+    t1 = __shfl_xor_sync(hmask, mx, 4);
+    mx = t1 > mx ? t1 : mx;
+    t1 = __shfl_xor_sync(hmask, mx, 8);
+    mx = t1 > mx ? t1 : mx;
     const double thresh = fmax(10.0 * DBL_EPSILON * bits_double(mx), DBL_MIN);
     const unsigned long long tb = abs_bits(thresh);
-    double X[4];
-    if (!sylv22_regs(D, X)) { *fallback = true; return false; }
-    // reflector 1 on column 0 of [-X; I]: (-x00, -x10, 1, 0)
-    const double a0 = -X[0], x1 = -X[1];
-    const double sig1 = fma(x1, x1, 1.0);
-    const double n1 = sqrt(fma(a0, a0, sig1));
-    const double be1 = a0 >= 0.0 ? -n1 : n1;
-    const double d1 = a0 - be1, rd1 = 1.0 / d1;
-    const double v10 = 1.0, v11 = x1 * rd1, v12 = rd1;  // v13 = 0
-    const double t1 = -d1 / be1;
-    // H1 applied to column 1 of [-X; I]: (-x01, -x11, 0, 1)
-    const double m0 = -X[2], m1 = -X[3], m2 = 0.0, m3 = 1.0;
-    const double w1 = fma(v12, m2, fma(v11, m1, v10 * m0)) * t1;
-    const double q1 = fma(-w1, v11, m1), q2 = fma(-w1, v12, m2), q3 = m3;
-    (void)m0;
-    // reflector 2 on (q1, q2, q3)
-    const double sig2 = fma(q3, q3, q2 * q2);
-    double u1 = 1.0, u2 = 0.0, u3 = 0.0, t2 = 0.0;
-    if (sig2 != 0.0) {
-        const double n2 = sqrt(fma(q1, q1, sig2));
-        const double be2 = q1 >= 0.0 ? -n2 : n2;
-        const double d2 = q1 - be2, rd2 = 1.0 / d2;
-        u2 = q2 * rd2;
-        u3 = q3 * rd2;
-        t2 = -d2 / be2;
+    // FP32 copies, scaled by the power of two of the largest entry of A and B
+    int em = 0;
+    {
+        auto up = [&](double v) {
+            const int e = (__double2hiint(v) >> 20) & 0x7ff;
+            em = e > em ? e : em;
+        };
+        up(a00); up(a10); up(a01); up(a11); up(b10); up(b01); up(b11);
     }
-    // Qs = (I - t1 v v^T)(I - t2 u u^T), v = (1, v11, v12, 0), u = (0, 1, u2, u3)
-    const double vu = fma(v12, u2, v11 * u1);
-    const double vr = sel4(r, v10, v11, v12, 0.0), vc = sel4(c, v10, v11, v12, 0.0);
-    const double ur = sel4(r, 0.0, u1, u2, u3), uc = sel4(c, 0.0, u1, u2, u3);
-    double qs = (r == c) ? 1.0 : 0.0;
-    qs = fma(-t1 * vr, vc, qs);
-    qs = fma(-t2 * ur, uc, qs);
-    qs = fma(t1 * t2 * vu * vr, uc, qs);
+    const int eoff = em - 127;
+    const float fa00 = to_f32(a00, eoff), fa01 = to_f32(a01, eoff), fa10 = to_f32(a10, eoff);
+    const float fa11 = to_f32(a11, eoff), fb01 = to_f32(b01, eoff), fb10 = to_f32(b10, eoff);
+    const float tr = to_f32(b11, eoff);
+    const float com = fmaf(fa01, fa10, -fb01 * fb10), rest = fa00 + fa11 - tr;
+    const float m00 = fmaf(fa00, fa00 - tr, com), m11 = fmaf(fa11, fa11 - tr, com);
+    const float m01 = fa01 * rest, m10 = fa10 * rest;
+    const float rdet = __fdividef(1.0f, fmaf(m00, m11, -m01 * m10));
+    float x[4];  // X column by column
+    auto solve = [&](float r00, float r10, float r01, float r11) {
+        const float y00 = fmaf(fa00 - tr, r00, fmaf(fa01, r10, fb10 * r01));
+        const float y10 = fmaf(fa11 - tr, r10, fmaf(fa10, r00, fb10 * r11));
+        const float y01 = fmaf(fa00, r01, fmaf(fa01, r11, fb01 * r00));
+        const float y11 = fmaf(fa11, r11, fmaf(fa10, r01, fb01 * r10));
+        x[0] = fmaf(m11, y00, -m01 * y10) * rdet;
+        x[1] = fmaf(m00, y10, -m10 * y00) * rdet;
+        x[2] = fmaf(m11, y01, -m01 * y11) * rdet;
+        x[3] = fmaf(m00, y11, -m10 * y01) * rdet;
+        return fmaxf(fmaxf(fabsf(x[0]), fabsf(x[1])), fmaxf(fabsf(x[2]), fabsf(x[3])));
+    };
+    // lane's entry (i, k) of the 2x2 matrices X and of the residual
+    const int i = l & 1, k = (l >> 1) & 1;
+    const double ai0 = i ? a10 : a00, ai1 = i ? a11 : a01;
+    const double bk0 = k ? b01 : 0.0, bk1 = k ? b11 : b10;
+    const double cik = Sp[poff(ja + 2 + k) + ja + i];
+    double X[4], own = cik;
+    float xmax = 0.0f;
+    bool good = false;
+    auto spread = [&](float v) {  // entries (0,0), (1,0), (0,1), (1,1) of the lanes
+        return solve(__shfl_sync(hmask, v, hbase), __shfl_sync(hmask, v, hbase + 1),
+                     __shfl_sync(hmask, v, hbase + 2), __shfl_sync(hmask, v, hbase + 3));
+    };
+    xmax = spread(to_f32(cik, eoff));
+    own = from_f32(k ? (i ? x[3] : x[2]) : (i ? x[1] : x[0]));
+#pragma unroll 1
+    for (int it = 0; it < 6; ++it) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) X[t] = __shfl_sync(hmask, own, hbase + t);
+        double res = fma(-ai0, k ? X[2] : X[0], cik);
+        res = fma(-ai1, k ? X[3] : X[1], res);
+        res = fma(i ? X[1] : X[0], bk0, res);
+        res = fma(i ? X[3] : X[2], bk1, res);
+        const float dmax = spread(to_f32(res, eoff));
+        own += from_f32(k ? (i ? x[3] : x[2]) : (i ? x[1] : x[0]));
+        if (!(dmax <= 0.25f * xmax)) break;  // also NaN: no convergence
+        if (it > 0 && dmax <= 1.4551915e-11f * xmax) { good = xmax < 1e30f; break; }
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) X[t] = __shfl_sync(hmask, own, hbase + t);
+    if (!good) {
+        double Xf[4];
+        if (!sylv22_full(Sp, ja, Xf)) return false;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) X[t] = Xf[t];
+    }
+    // reflector 1 on column 0 of [-X; I], (-x00, -x10, 1, 0); reflector 2 on
+    // rows 1..3 of reflector 1 times column 1, (-x01, -x11, 0, 1)
+    const double w1 = -X[1];
+    double w0, f1, u0, f2;
+    refl3(-X[0], w1, &w0, &f1);
+    const double s1 = fma(w0, -X[2], w1 * -X[3]) * f1;
+    const double q1 = fma(-s1, w1, -X[3]), u1 = -s1;  // (q1, u1, 1)
+    refl3(q1, u1, &u0, &f2);
+    // Qs = (I - f1 w w^T)(I - f2 u u^T), w = (w0, w1, 1, 0), u = (0, u0, u1, 1)
+    const double wu = fma(w1, u0, u1);
+    const double wr = sel4(r, w0, w1, 1.0, 0.0), wc = sel4(c, w0, w1, 1.0, 0.0);
+    const double ur = sel4(r, 0.0, u0, u1, 1.0), uc = sel4(c, 0.0, u0, u1, 1.0);
+    const double ar = f1 * wr;
+    double qs = fma(-ar, wc, (r == c) ? 1.0 : 0.0);
+    qs = fma(-(f2 * uc), fma(-ar, wu, ur), qs);
     // T = Qs^T D: T[r][c] = sum_a Qs[a][r] D[a][c]
-    double dcol0 = sel4(c, D[0], D[4], D[8], D[12]), dcol1 = sel4(c, D[1], D[5], D[9], D[13]);
-    double dcol2 = sel4(c, D[2], D[6], D[10], D[14]), dcol3 = sel4(c, D[3], D[7], D[11], D[15]);
-    double T = 0.0;
-    T = fma(__shfl_sync(hmask, qs, hbase + 0 + 4 * r), dcol0, T);
-    T = fma(__shfl_sync(hmask, qs, hbase + 1 + 4 * r), dcol1, T);
-    T = fma(__shfl_sync(hmask, qs, hbase + 2 + 4 * r), dcol2, T);
-    T = fma(__shfl_sync(hmask, qs, hbase + 3 + 4 * r), dcol3, T);
+    double T = __shfl_sync(hmask, qs, hbase + 0 + 4 * r) * dc0;
+    T = fma(__shfl_sync(hmask, qs, hbase + 1 + 4 * r), dc1, T);
+    T = fma(__shfl_sync(hmask, qs, hbase + 2 + 4 * r), dc2, T);
+    T = fma(__shfl_sync(hmask, qs, hbase + 3 + 4 * r), dc3, T);
     // Dt = T Qs: Dt[r][c] = sum_b T[r][b] Qs[b][c]
     double Dt = 0.0;
 #pragma unroll
@@ -221,7 +369,7 @@ __device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, i
     // weak test on the lower-left 2x2 block
     const bool low = (r >= 2 && c < 2);
     const bool weak_bad = low && abs_bits(Dt) > tb;
-    if (__any_sync(hmask, weak_bad)) { *fallback = true; return false; }
+    if (__any_sync(hmask, weak_bad)) return false;
     const double Dt0 = low ? 0.0 : Dt;
     if (strong) {
         // P = Qs Dt0: P[r][b] = sum_a Qs[r][a] Dt0[a][b]
@@ -236,13 +384,121 @@ __device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, i
         for (int bb = 0; bb < 4; ++bb)
             E = fma(__shfl_sync(hmask, P, hbase + r + 4 * bb), __shfl_sync(hmask, qs, hbase + c + 4 * bb),
                     E);
-        const double drc = sel4(r, dcol0, dcol1, dcol2, dcol3);
-        E -= drc;
-        if (__any_sync(hmask, abs_bits(E) > tb)) { *fallback = true; return false; }
+        E -= sel4(r, dc0, dc1, dc2, dc3);
+        if (__any_sync(hmask, abs_bits(E) > tb)) return false;
     }
-    *zrc = qs;
+    z[0] = w0;
+    z[1] = w1;
+    z[2] = f1;
+    z[3] = u0;
+    z[4] = u1;
+    z[5] = f2;
     *dnrc = Dt0;
     return true;
+}
+
+// k = 3 swap by four lanes (all 32 lanes of the warp call it, eight swaps at a
+// time; base is the first lane of the quad, q this lane in it).  2|1:
+// D = [[A, c], [0, lam]] with A 2x2; X solves (A - lam I) X = c, and the one
+// reflector H with H (-x0, -x1, 1)^T = beta e_0 gives H D H with lam first.
+// 1|2 is the same on the flipped block F D^T F (F reverses the indices).
+// Lane q < 3 owns column q of the block, and row q after the exchange between
+// the two products.  The result: z = (w0, w1, f) of the reflector (in flipped
+// index order if flip), dn = row q of the new (flipped) block.  Returns
+// false, for all four lanes, when this path cannot decide (tiny pivot) or
+// the swap fails the weak or strong test.  52 FP64 instructions; one lane per
+// swap, with CUDA's divisions and square root, took about 140.
+__device__ __forceinline__ bool swap3_quad(const double* __restrict__ Sp, int ja, bool flip, int q,
+                                           int base, bool strong, double* z, double* dn) {
+    const unsigned full = 0xffffffffu;
+    const double* c0 = Sp + poff(ja) + ja;
+    const double* c1 = Sp + poff(ja + 1) + ja;
+    const double* c2 = Sp + poff(ja + 2) + ja;
+    // flipped entry (r, c) is entry (2 - c, 2 - r)
+    const double d00 = flip ? c2[2] : c0[0], d10 = flip ? c1[2] : c0[1];
+    const double d01 = flip ? c2[1] : c1[0], d11 = c1[1];
+    const double d02 = c2[0], d12 = flip ? c1[0] : c2[1], lam = flip ? c0[0] : c2[2];
+    unsigned long long mx = abs_bits(d00);
+    auto up = [](unsigned long long& m, double v) {
+        const unsigned long long b = abs_bits(v);
+        m = b > m ? b : m;
+    };
+    up(mx, d10); up(mx, d01); up(mx, d11); up(mx, d02); up(mx, d12); up(mx, lam);
+    const double thresh = fmax(10.0 * DBL_EPSILON * bits_double(mx), DBL_MIN);
+    const unsigned long long tb = abs_bits(thresh);
+    const double a00 = d00 - lam, a11 = d11 - lam;
+    const double det = fma(a00, a11, -(d01 * d10));
+    // |det| must not be tiny against the entries
+    unsigned long long am = abs_bits(a00);
+    up(am, d01); up(am, d10); up(am, a11);
+    const double amax = bits_double(am);
+    bool ok = abs_bits(det) > abs_bits(1e-4 * amax * amax);
+    const double rdet = rcp64(ok ? det : 1.0);
+    // lane 1 of the quad computes x1, the others x0
+    const double xo = fma(q == 1 ? a00 : a11, q == 1 ? d12 : d02, -((q == 1 ? d10 : d01) * (q == 1 ? d02 : d12))) *
+                      rdet;
+    const double x0 = __shfl_sync(full, xo, base), w1 = -__shfl_sync(full, xo, base + 1);
+    double w0, f;
+    refl3(-x0, w1, &w0, &f);
+    // column q of H D
+    double t0 = q == 0 ? d00 : (q == 1 ? d01 : d02), t1 = q == 0 ? d10 : (q == 1 ? d11 : d12);
+    double t2 = q >= 2 ? lam : 0.0;
+    const double s0 = t0, s1 = t1, s2 = t2;  // column q of D
+    apply_refl3(w0, w1, f, &t0, &t1, &t2);
+    // 3x3 transposition within the quad (lane 3 mirrors lane 2)
+    auto flip3 = [&](double& v0, double& v1, double& v2) {
+        const double a0 = __shfl_sync(full, v0, base), a1 = __shfl_sync(full, v1, base);
+        const double a2 = __shfl_sync(full, v2, base), b0 = __shfl_sync(full, v0, base + 1);
+        const double b1 = __shfl_sync(full, v1, base + 1), b2 = __shfl_sync(full, v2, base + 1);
+        const double e0 = __shfl_sync(full, v0, base + 2), e1 = __shfl_sync(full, v1, base + 2);
+        const double e2 = __shfl_sync(full, v2, base + 2);
+        v0 = q == 0 ? a0 : (q == 1 ? a1 : a2);
+        v1 = q == 0 ? b0 : (q == 1 ? b1 : b2);
+        v2 = q == 0 ? e0 : (q == 1 ? e1 : e2);
+    };
+    flip3(t0, t1, t2);                      // row q of H D
+    apply_refl3(w0, w1, f, &t0, &t1, &t2);  // row q of H D H
+    // weak test: rows 1 and 2 of column 0 must vanish
+    if (q > 0) {
+        ok = ok && abs_bits(t0) <= tb;
+        t0 = 0.0;
+    }
+    dn[0] = t0;
+    dn[1] = t1;
+    dn[2] = t2;
+    if (strong) {
+        apply_refl3(w0, w1, f, &t0, &t1, &t2);  // row q of Dt0 H
+        flip3(t0, t1, t2);                      // column q of it
+        apply_refl3(w0, w1, f, &t0, &t1, &t2);
+        ok = ok && abs_bits(t0 - s0) <= tb && abs_bits(t1 - s1) <= tb && abs_bits(t2 - s2) <= tb;
+    }
+    z[0] = w0;
+    z[1] = w1;
+    z[2] = f;
+    const unsigned votes = __ballot_sync(full, ok);
+    return ((votes >> base) & 15u) == 15u;
+}
+
+// Givens rotation (c, s) from (t, d): (t, d) / |(t, d)|.  Values whose squares
+// leave the normal range are scaled by a power of two first.
+__device__ __forceinline__ void givens64(double t, double d, double* c, double* s) {
+    double nn = fma(t, t, d * d);
+    const unsigned e = (unsigned)__double2hiint(nn) >> 20;
+    if (e < 100u || e > 1900u) {
+        const unsigned long long bt = abs_bits(t), bd = abs_bits(d);
+        const int em = (int)((bt > bd ? bt : bd) >> 52);
+        const double sc = __hiloint2double((em < 1 ? 2045 : (em > 2045 ? 1 : 2046 - em)) << 20, 0);
+        t *= sc;
+        d *= sc;
+        nn = fma(t, t, d * d);
+    }
+    // 1 / sqrt(nn): one third-order step, y (1 + e/2 + 3 e^2 / 8) with
+    // e = 1 - nn y^2 (the binomial series of (1 - e)^(-1/2))
+    const double y = rsqrt_seed(nn);
+    const double r = fma(-(nn * y), y, 1.0);
+    const double rh = fma(y * r, fma(0.375, r, 0.5), y);
+    *c = t * rh;
+    *s = d * rh;
 }
 
 // Swap types of a step, each handled by its own warps (FP64 issue costs the
@@ -310,61 +566,73 @@ constexpr size_t kWindowSmem = sizeof(double) * ((size_t)WMAX * WMAX +
 constexpr size_t kWindowSmemWide = sizeof(double) * (size_t)2 * (WMAX_WIDE / 2) * 16 +
                                    sizeof(int) * 2 * 3 * (WMAX_WIDE / 2) + 2 * WMAX_WIDE;
 
-// Row r of U, columns [j, j + K) <- (those columns) Z (the right
-// transformation of one swap, applied to U).
+// How a step's slot keeps its transformation Z (swk[slot] = k, plus Z_MATRIX
+// where the full transform computed it; swp[slot] tells 1|2 from 2|1):
+//   k = 2: Z = [[c, -s], [s, c]] as (c, s);
+//   k = 3: one reflector (w0, w1, f), in reversed index order for 1|2;
+//   k = 4: two reflectors (w0, w1, f) on 0..2 and (u0, u1, f') on 1..3;
+//   Z_MATRIX: the k x k matrix, column-major with leading dimension 4.
+// The reflectors take 6 and 12 FP64 instructions per row where the matrices
+// take 9 and 16.
+constexpr int Z_MATRIX = 16;
+
+// x <- x Z for one row x of K values (or Z^T x for a column).
 template <int K>
-__device__ __forceinline__ void right_u_row(double* __restrict__ U, int w, int j, int r,
-                                            const double* __restrict__ Z) {
-    double x[K], y[K];
+__device__ __forceinline__ void apply_z(const double* __restrict__ Z, bool matrix, double* x) {
+    if constexpr (K == 2) {
+        const double c = Z[0], s = Z[1];
+        const double y = fma(s, x[1], c * x[0]);
+        x[1] = fma(c, x[1], -(s * x[0]));
+        x[0] = y;
+    } else {
+        if (matrix) {
+            double y[K];
 #pragma unroll
-    for (int i = 0; i < K; ++i) x[i] = U[(j + i) * w + r];
+            for (int c = 0; c < K; ++c) {
+                double acc = 0.0;
 #pragma unroll
-    for (int c = 0; c < K; ++c) {
-        double acc = 0.0;
+                for (int i = 0; i < K; ++i) acc = fma(x[i], Z[c * 4 + i], acc);
+                y[c] = acc;
+            }
 #pragma unroll
-        for (int i = 0; i < K; ++i) acc = fma(x[i], Z[c * 4 + i], acc);
-        y[c] = acc;
+            for (int c = 0; c < K; ++c) x[c] = y[c];
+        } else {
+            apply_refl3(Z[0], Z[1], Z[2], &x[0], &x[1], &x[2]);
+            if constexpr (K == 4) apply_refl3(Z[3], Z[4], Z[5], &x[1], &x[2], &x[3]);
+        }
     }
-#pragma unroll
-    for (int c = 0; c < K; ++c) U[(j + c) * w + r] = y[c];
 }
 
-// Left transformation of one swap on one column c of the packed window:
-// rows [j, j + K) of column c <- Z^T (those rows).
+// The slot's transformation on K values x0[0], x0[stride(1)], ...: rows
+// [j, j + K) of a column of the packed window (left), columns [j, j + K) of a
+// row of it or of U (right).  at(i) is the address of the i-th value.
+template <int K, typename At>
+__device__ __forceinline__ void apply_slot(const double* __restrict__ Z, int kk, int p, At at) {
+    const bool matrix = K > 2 && (kk & Z_MATRIX);
+    const bool flip = K == 3 && p == 1 && !matrix;
+    double x[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) x[i] = *at(K == 3 && flip ? K - 1 - i : i);
+    apply_z<K>(Z, matrix, x);
+#pragma unroll
+    for (int i = 0; i < K; ++i) *at(K == 3 && flip ? K - 1 - i : i) = x[i];
+}
 template <int K>
 __device__ __forceinline__ void left_col(double* __restrict__ Sp, int j, int c,
-                                         const double* __restrict__ Z) {
-    double x[K], y[K];
-#pragma unroll
-    for (int r = 0; r < K; ++r) x[r] = Sp[poff(c) + j + r];
-#pragma unroll
-    for (int r = 0; r < K; ++r) {
-        double acc = 0.0;
-#pragma unroll
-        for (int i = 0; i < K; ++i) acc = fma(Z[r * 4 + i], x[i], acc);
-        y[r] = acc;
-    }
-#pragma unroll
-    for (int r = 0; r < K; ++r) Sp[poff(c) + j + r] = y[r];
+                                         const double* __restrict__ Z, int kk, int p) {
+    double* x = Sp + poff(c) + j;
+    apply_slot<K>(Z, kk, p, [&](int i) { return x + i; });
 }
-
-// Right transformation of one swap on one row r (< j) of the packed window:
-// columns [j, j + K) of row r <- (those columns) Z.
 template <int K>
 __device__ __forceinline__ void right_row(double* __restrict__ Sp, int j, int r,
-                                          const double* __restrict__ Z) {
-    double x[K], y[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i) x[i] = Sp[poff(j + i) + r];
-#pragma unroll
-    for (int c = 0; c < K; ++c) {
-        double acc = 0.0;
-#pragma unroll
-        for (int i = 0; i < K; ++i) acc = fma(x[i], Z[c * 4 + i], acc);
-        y[c] = acc;
-    }
-#pragma unroll
-    for (int c = 0; c < K; ++c) Sp[poff(j + c) + r] = y[c];
+                                          const double* __restrict__ Z, int kk, int p) {
+    apply_slot<K>(Z, kk, p, [&](int i) { return Sp + poff(j + i) + r; });
+}
+template <int K>
+__device__ __forceinline__ void right_u_row(double* __restrict__ U, int w, int j, int r,
+                                            const double* __restrict__ Z, int kk, int p) {
+    double* x = U + j * w + r;
+    apply_slot<K>(Z, kk, p, [&](int i) { return x + i * w; });
 }
 
 // Last i in [0, cnt) with pre[i] <= it (pre is nondecreasing, pre[0] = 0).
@@ -438,7 +706,6 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
     constexpr int MSW = WM / 2;  // at most one swap per two positions
     constexpr int NTW = WIN_TWARPS;
     static_assert(NTW % 4 == 0 && NTW < WIN_THREADS / 32, "transform warps per sub-partition");
-    constexpr int PTHREADS = WIN_THREADS - 32 * NTW;
     double* U = WIDE ? Ug : reinterpret_cast<double*>(smem_raw);        // w*w
     double* Sp = WIDE ? gsp : U + WM * WM;                               // packed window
     double* Zbuf = WIDE ? reinterpret_cast<double*>(smem_raw) : Sp + poff(WM);  // [2][MSW * 16]
@@ -602,6 +869,7 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                 sel[swp[sw]] = SEL_STUCK;
                 continue;
             }
+            k &= Z_MATRIX - 1;
             // in-window flops of this accepted transform: k x k applied to
             // w - j - k columns (left) and j rows of S + its U rows (right)
             wflops += 2ull * k * k *
@@ -621,10 +889,10 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
     };
 
     // --- phase A2 of the step of parity pi, by the transform warps (warps
-    // 0 .. NTW - 1, NTW / 4 per sub-partition; type-uniform, since an FP64
-    // issue costs the same for 1 or 32 active lanes): 2|2 swaps on
-    // sub-partitions 0 and 1 (one per half-warp), k = 3 on 2, 1|1 rotations
-    // on 3.
+    // 0 .. NTW - 1, NTW / 4 per sub-partition).  An FP64 instruction costs the
+    // same for 1 or 32 active lanes, so a warp takes swaps of one type at a
+    // time, as many as its lanes hold: two 2|2 swaps, eight k = 3 swaps or 32
+    // rotations, dealt out in this order (the longest chains first).
     auto transforms = [&](int pi) {
         double* Zs = Zbuf + pi * MSW * 16;
         int* swj = swbuf + pi * 3 * MSW;
@@ -632,104 +900,119 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
         int* swp = swk + MSW;
         const int (*tlist)[MSW] = tlist2[pi];
         const int* tcnt = tcnt2[pi];
-        const int part = warp & 3, rank = warp >> 2;
-        constexpr int NRANK = NTW / 4;
-        const int ty = part <= 1 ? T_22 : (part == 2 ? T_3 : T_11);
-        if (ty == T_22) {
-            // two 2|2 swaps per warp, one per half-warp
-            const int h = lane >> 4, l = lane & 15;
-            const unsigned hmask = h ? 0xffff0000u : 0x0000ffffu;
-            for (int i = (rank * 2 + part) * 2 + h; i < tcnt[T_22]; i += 4 * NRANK) {
-                const int slot = tlist[T_22][i];
-                const int ja = swj[slot];
-                double zrc = 0.0, dnrc = 0.0;
-                bool fb = false;
-                bool ok = swap22_halfwarp(Sp, ja, l, hmask, h * 16, strong != 0, &zrc, &dnrc, &fb);
-                const int r = l & 3, c = l >> 2;
-                if (ok) {
-                    Zs[slot * 16 + c * 4 + r] = zrc;
-                    if (r <= c + 1) Sp[poff(ja + c) + ja + r] = dnrc;
-                    if (l == 0) atomicAdd(&nacc, 1);
-                } else if (l == 0) {
-                    double D[16], Zl[16], Dn[16];
-                    for (int cc = 0; cc < 4; ++cc)
-                        for (int rr = 0; rr < 4; ++rr)
-                            D[cc * 4 + rr] = (rr <= cc + 1) ? Sp[poff(ja + cc) + ja + rr] : 0.0;
-                    if (swap_transform(D, 2, 2, strong != 0, Zl, Dn)) {
-                        for (int cc = 0; cc < 4; ++cc)
-                            for (int rr = 0; rr <= min(cc + 1, 3); ++rr)
-                                Sp[poff(ja + cc) + ja + rr] = Dn[cc * 4 + rr];
-                        for (int e = 0; e < 16; ++e) Zs[slot * 16 + e] = Zl[e];
-                        atomicAdd(&nacc, 1);
-                    } else {
-                        swk[slot] = 0;
-                        swp[slot] = ja + 2;
-                        atomicAdd(&nrej, 1);
-                    }
-                }
-                __syncwarp(hmask);
-            }
-            return;
-        }
-        for (int i = rank * 32 + lane; i < tcnt[ty]; i += 32 * NRANK) {
-            const int slot = tlist[ty][i];
-            const int ja = swj[slot], p = swp[slot], k = swk[slot], q = k - p;
-            double* Z = &Zs[slot * 16];
-            bool ok;
-            if (ty == T_11 && p < 0) {
-                // restore the standard form of the 2x2 block at ja
-                double m[16];
-                m[0] = Sp[poff(ja) + ja];
-                m[1] = Sp[poff(ja) + ja + 1];
-                m[4] = Sp[poff(ja + 1) + ja];
-                m[5] = Sp[poff(ja + 1) + ja + 1];
-                double cs, sn;
-                standardize2(m, &cs, &sn);
-                Sp[poff(ja) + ja] = m[0];
-                Sp[poff(ja) + ja + 1] = m[1];
-                Sp[poff(ja + 1) + ja] = m[4];
-                Sp[poff(ja + 1) + ja + 1] = m[5];
-                Z[0] = cs; Z[1] = sn; Z[4] = -sn; Z[5] = cs;
-                ok = true;
-            } else if (ty == T_11) {
-                // Givens rotation from (t12, t22 - t11); always accepted
-                double t11 = Sp[poff(ja) + ja], t12 = Sp[poff(ja + 1) + ja];
-                double t22 = Sp[poff(ja + 1) + ja + 1];
-                double c = 1.0, sn = 0.0, n12 = t12;
-                if (t11 != t22) {
-                    double d = t22 - t11;
-                    double rh = 1.0 / sqrt(fma(t12, t12, d * d));
-                    c = t12 * rh;
-                    sn = d * rh;
-                    double r12 = fma(c, t12, sn * t22);
-                    n12 = fma(r12, c, -(c * t11) * sn);
-                }
-                Z[0] = c; Z[1] = sn; Z[4] = -sn; Z[5] = c;
-                Sp[poff(ja) + ja] = t22;
-                Sp[poff(ja) + ja + 1] = 0.0;
-                Sp[poff(ja + 1) + ja] = n12;
-                Sp[poff(ja + 1) + ja + 1] = t11;
-                ok = true;
-            } else {
-                double D[16], Zl[16], Dn[16];
-                for (int cc = 0; cc < 3; ++cc)
-                    for (int rr = 0; rr < 3; ++rr)
-                        D[cc * 4 + rr] = (rr <= cc + 1) ? Sp[poff(ja + cc) + ja + rr] : 0.0;
-                ok = swap3_fast(D, p, strong != 0, Zl, Dn) ||
-                     swap_transform(D, p, q, strong != 0, Zl, Dn);
-                if (ok) {
-                    for (int cc = 0; cc < 3; ++cc)
-                        for (int rr = 0; rr <= min(cc + 1, 2); ++rr)
-                            Sp[poff(ja + cc) + ja + rr] = Dn[cc * 4 + rr];
-                    for (int e = 0; e < 16; ++e) Z[e] = Zl[e];
-                }
-            }
-            if (ok) {
-                if (p >= 0) atomicAdd(&nacc, 1);
+        const int n22 = (tcnt[T_22] + 1) >> 1, n3 = (tcnt[T_3] + 7) >> 3;
+        const int nunits = n22 + n3 + ((tcnt[T_11] + 31) >> 5);
+        // the full transform of a swap, by one lane
+        auto full = [&](int slot) {
+            const int ja = swj[slot], p = swp[slot], k = swk[slot];
+            double D[16], Zl[16], Dn[16];
+            for (int cc = 0; cc < k; ++cc)
+                for (int rr = 0; rr < k; ++rr)
+                    D[cc * 4 + rr] = (rr <= cc + 1) ? Sp[poff(ja + cc) + ja + rr] : 0.0;
+            if (swap_transform(D, p, k - p, strong != 0, Zl, Dn)) {
+                for (int cc = 0; cc < k; ++cc)
+                    for (int rr = 0; rr <= min(cc + 1, k - 1); ++rr)
+                        Sp[poff(ja + cc) + ja + rr] = Dn[cc * 4 + rr];
+                for (int e = 0; e < 16; ++e) Zs[slot * 16 + e] = Zl[e];
+                swk[slot] = k | Z_MATRIX;
+                atomicAdd(&nacc, 1);
             } else {
                 swk[slot] = 0;
                 swp[slot] = ja + p;   // the stuck (selected) block
                 atomicAdd(&nrej, 1);
+            }
+        };
+        for (int u = warp; u < nunits; u += NTW) {
+            if (u < n22) {
+                // two 2|2 swaps, one per half-warp
+                const int h = lane >> 4, l = lane & 15, i = 2 * u + h;
+                const unsigned hmask = h ? 0xffff0000u : 0x0000ffffu;
+                if (i < tcnt[T_22]) {
+                    const int slot = tlist[T_22][i];
+                    const int ja = swj[slot];
+                    double z[6], dnrc = 0.0;
+                    const bool ok = swap22_halfwarp(Sp, ja, l, hmask, h * 16, strong != 0, z, &dnrc);
+                    const int r = l & 3, c = l >> 2;
+                    if (ok) {
+                        if (r <= c + 1) Sp[poff(ja + c) + ja + r] = dnrc;
+                        if (l == 0) {
+#pragma unroll
+                            for (int e = 0; e < 6; ++e) Zs[slot * 16 + e] = z[e];
+                            atomicAdd(&nacc, 1);
+                        }
+                    } else if (l == 0) {
+                        full(slot);
+                    }
+                }
+                __syncwarp();
+            } else if (u < n22 + n3) {
+                // eight k = 3 swaps, one per quad of lanes
+                const int q = lane & 3, i = 8 * (u - n22) + (lane >> 2);
+                const bool act = i < tcnt[T_3];
+                const int slot = tlist[T_3][act ? i : tcnt[T_3] - 1];
+                const int ja = swj[slot];
+                const bool flip = swp[slot] == 1;
+                double z[3], dn[3];
+                const bool ok = swap3_quad(Sp, ja, flip, q, lane & ~3, strong != 0, z, dn);
+                __syncwarp();
+                if (act && ok) {
+                    // row q of the flipped block: entry (q, c) is (2 - c, 2 - q)
+                    if (q < 3)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const int rr = flip ? 2 - c : q, cc = flip ? 2 - q : c;
+                            if (rr <= cc + 1) Sp[poff(ja + cc) + ja + rr] = dn[c];
+                        }
+                    if (q == 0) {
+                        Zs[slot * 16] = z[0];
+                        Zs[slot * 16 + 1] = z[1];
+                        Zs[slot * 16 + 2] = z[2];
+                        atomicAdd(&nacc, 1);
+                    }
+                } else if (act && q == 0) {
+                    full(slot);
+                }
+                __syncwarp();
+            } else {
+                // 32 rotations
+                const int i = 32 * (u - n22 - n3) + lane;
+                if (i < tcnt[T_11]) {
+                    const int slot = tlist[T_11][i];
+                    const int ja = swj[slot], p = swp[slot];
+                    double* Z = &Zs[slot * 16];
+                    double* c0 = Sp + poff(ja) + ja;
+                    double* c1 = Sp + poff(ja + 1) + ja;
+                    if (p < 0) {
+                        // restore the standard form of the 2x2 block at ja
+                        double m[16];
+                        m[0] = c0[0];
+                        m[1] = c0[1];
+                        m[4] = c1[0];
+                        m[5] = c1[1];
+                        double cs, sn;
+                        standardize2(m, &cs, &sn);
+                        c0[0] = m[0];
+                        c0[1] = m[1];
+                        c1[0] = m[4];
+                        c1[1] = m[5];
+                        Z[0] = cs;
+                        Z[1] = sn;
+                    } else {
+                        // Givens rotation from (t12, t22 - t11), always
+                        // accepted; t12 stays (the norm of the block and of
+                        // its diagonal do)
+                        const double t11 = c0[0], t12 = c1[0], t22 = c1[1];
+                        double c = 1.0, sn = 0.0;
+                        if (t11 != t22) givens64(t12, t22 - t11, &c, &sn);
+                        Z[0] = c;
+                        Z[1] = sn;
+                        c0[0] = t22;
+                        c0[1] = 0.0;
+                        c1[1] = t11;
+                        atomicAdd(&nacc, 1);
+                    }
+                }
+                __syncwarp();
             }
         }
     };
@@ -749,6 +1032,7 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
         const double* Zs = Zbuf + pp * MSW * 16;
         const int* swj = swbuf + pp * 3 * MSW;
         const int* swk = swj + MSW;
+        const int* swp = swk + MSW;
         const int (*tlist)[MSW] = tlist2[pp];
         const int* tcnt = tcnt2[pp];
         constexpr int NCL = CRIT_L - 2, NCR = CRIT_R - 2;  // item slots per swap
@@ -765,13 +1049,14 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                 for (int it = claim(0, g); it - lane < total; it = claim(0, g)) {
                     if (it >= total) continue;
                     const int slot = tlist[g][it / NCL];
-                    if (swk[slot] == 0) continue;  // rejected
+                    const int kk = swk[slot];
+                    if (kk == 0) continue;  // rejected
                     const int j = swj[slot], c = j + k + it % NCL;
                     if (c >= min(w, j + CRIT_L)) continue;
                     const double* Z = Zs + slot * 16;
-                    if (g == 0) left_col<2>(Sp, j, c, Z);
-                    else if (g == 1) left_col<3>(Sp, j, c, Z);
-                    else left_col<4>(Sp, j, c, Z);
+                    if (g == 0) left_col<2>(Sp, j, c, Z, kk, swp[slot]);
+                    else if (g == 1) left_col<3>(Sp, j, c, Z, kk, swp[slot]);
+                    else left_col<4>(Sp, j, c, Z, kk, swp[slot]);
                 }
             }
         }
@@ -783,13 +1068,14 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                 for (int it = claim(1, g); it - lane < total; it = claim(1, g)) {
                     if (it >= total) continue;
                     const int slot = tlist[g][it / NCR];
-                    if (swk[slot] == 0) continue;
+                    const int kk = swk[slot];
+                    if (kk == 0) continue;
                     const int j = swj[slot], r = j - 1 - it % NCR;
                     if (r < max(0, j + k - CRIT_R)) continue;
                     const double* Z = Zs + slot * 16;
-                    if (g == 0) right_row<2>(Sp, j, r, Z);
-                    else if (g == 1) right_row<3>(Sp, j, r, Z);
-                    else right_row<4>(Sp, j, r, Z);
+                    if (g == 0) right_row<2>(Sp, j, r, Z, kk, swp[slot]);
+                    else if (g == 1) right_row<3>(Sp, j, r, Z, kk, swp[slot]);
+                    else right_row<4>(Sp, j, r, Z, kk, swp[slot]);
                 }
             }
         }
@@ -805,12 +1091,13 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                     if (it >= total) continue;
                     const int lo = prefix_slot(pre, cnt, it);
                     const int slot = tlist[g][lo];
-                    if (swk[slot] == 0) continue;
+                    const int kk = swk[slot];
+                    if (kk == 0) continue;
                     const int j = swj[slot], c = j + CRIT_L + (it - pre[lo]);
                     const double* Z = Zs + slot * 16;
-                    if (g == 0) left_col<2>(Sp, j, c, Z);
-                    else if (g == 1) left_col<3>(Sp, j, c, Z);
-                    else left_col<4>(Sp, j, c, Z);
+                    if (g == 0) left_col<2>(Sp, j, c, Z, kk, swp[slot]);
+                    else if (g == 1) left_col<3>(Sp, j, c, Z, kk, swp[slot]);
+                    else left_col<4>(Sp, j, c, Z, kk, swp[slot]);
                 }
             }
         }
@@ -825,12 +1112,13 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                     if (it >= total) continue;
                     const int lo = prefix_slot(pre, cnt, it);
                     const int slot = tlist[g][lo];
-                    if (swk[slot] == 0) continue;
+                    const int kk = swk[slot];
+                    if (kk == 0) continue;
                     const int j = swj[slot], r = it - pre[lo];
                     const double* Z = Zs + slot * 16;
-                    if (g == 0) right_row<2>(Sp, j, r, Z);
-                    else if (g == 1) right_row<3>(Sp, j, r, Z);
-                    else right_row<4>(Sp, j, r, Z);
+                    if (g == 0) right_row<2>(Sp, j, r, Z, kk, swp[slot]);
+                    else if (g == 1) right_row<3>(Sp, j, r, Z, kk, swp[slot]);
+                    else right_row<4>(Sp, j, r, Z, kk, swp[slot]);
                 }
             }
 #pragma unroll
@@ -842,12 +1130,13 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                     if (it >= total) continue;
                     const int lo = prefix_slot(pre, cnt, it);
                     const int slot = tlist[g][lo];
-                    if (swk[slot] == 0) continue;
+                    const int kk = swk[slot];
+                    if (kk == 0) continue;
                     const int j = swj[slot], r = slo2[pp][slot] + (it - pre[lo]);
                     const double* Z = Zs + slot * 16;
-                    if (g == 0) right_u_row<2>(U, w, j, r, Z);
-                    else if (g == 1) right_u_row<3>(U, w, j, r, Z);
-                    else right_u_row<4>(U, w, j, r, Z);
+                    if (g == 0) right_u_row<2>(U, w, j, r, Z, kk, swp[slot]);
+                    else if (g == 1) right_u_row<3>(U, w, j, r, Z, kk, swp[slot]);
+                    else right_u_row<4>(U, w, j, r, Z, kk, swp[slot]);
                 }
             }
         }
