@@ -31,6 +31,8 @@
 #include <cuda_bf16.h>
 #include <float.h>
 
+#include <type_traits>
+
 namespace gbr {
 namespace win {
 
@@ -152,8 +154,9 @@ __device__ __forceinline__ bool sylv22_regs(const double* D, double* X) {
 // special function unit or from FP32, and FP64 only corrects them.  Measured
 // against transforms in FP64 throughout, with 3x3 and 4x4 products: a window
 // task of w = 128, m = 64 took 1.90 ms and takes 1.48 ms (median in the
-// n = 4000 schedule), one of w = 32, m = 16 took 268 us and takes 193 us; the
-// rounding errors of whole reorderings (orthogonality, residual, swaps sent to
+// n = 4000 schedule), one of w = 32, m = 16 took 268 us and took 193 us (1.31
+// ms and 145 us since the control of a step runs beside the critical products
+// and a lane of a product warp works on two items at once); the rounding errors of whole reorderings (orthogonality, residual, swaps sent to
 // the double-double retry) are a little smaller than they were.
 // ---------------------------------------------------------------------------
 // Seeds with about 20 correct bits (PTX rcp/rsqrt.approx.ftz.f64).
@@ -170,6 +173,17 @@ __device__ __forceinline__ double rsqrt_seed(double x) {
 // x times 2^-1 for a normal x above the smallest binade.
 __device__ __forceinline__ double half_of(double x) {
     return __longlong_as_double(__double_as_longlong(x) - (1LL << 52));
+}
+// x >= 0 and x == 0 (either zero) on the integer pipe.
+__device__ __forceinline__ bool nonneg(double x) {
+    return __double_as_longlong(x) >= 0 || __double_as_longlong(x) == (long long)(1ULL << 63);
+}
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+// max(10 eps m, DBL_MIN), the threshold of the stability tests, as a bit
+// pattern (m >= 0).
+__device__ __forceinline__ unsigned long long thresh_bits(unsigned long long m) {
+    const unsigned long long t = abs_bits(10.0 * DBL_EPSILON * bits_double(m));
+    return t > 0x0010000000000000ULL ? t : 0x0010000000000000ULL;
 }
 // 1/x for normal x: one third-order step, y (1 + e + e^2) with e = 1 - x y
 // (the geometric series of 1 / (1 - e)).
@@ -195,7 +209,7 @@ __device__ __forceinline__ double sqrt64(double x) {
 __device__ __forceinline__ void refl3(double a0, double a1, double* w0, double* f) {
     const double n1 = fma(a1, a1, 1.0);
     const double d = fabs(a0) + sqrt64(fma(a0, a0, n1));
-    *w0 = a0 >= 0.0 ? d : -d;
+    *w0 = nonneg(a0) ? d : -d;
     *f = rcp64(half_of(fma(d, d, n1)));
 }
 __device__ __forceinline__ void apply_refl3(double w0, double w1, double f, double* x0, double* x1,
@@ -274,8 +288,7 @@ __device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, i
     mx = t1 > mx ? t1 : mx;
     t1 = __shfl_xor_sync(hmask, mx, 8);
     mx = t1 > mx ? t1 : mx;
-    const double thresh = fmax(10.0 * DBL_EPSILON * bits_double(mx), DBL_MIN);
-    const unsigned long long tb = abs_bits(thresh);
+    const unsigned long long tb = thresh_bits(mx);
     // FP32 copies, scaled by the power of two of the largest entry of A and B
     int em = 0;
     {
@@ -424,8 +437,7 @@ __device__ __forceinline__ bool swap3_quad(const double* __restrict__ Sp, int ja
         m = b > m ? b : m;
     };
     up(mx, d10); up(mx, d01); up(mx, d11); up(mx, d02); up(mx, d12); up(mx, lam);
-    const double thresh = fmax(10.0 * DBL_EPSILON * bits_double(mx), DBL_MIN);
-    const unsigned long long tb = abs_bits(thresh);
+    const unsigned long long tb = thresh_bits(mx);
     const double a00 = d00 - lam, a11 = d11 - lam;
     const double det = fma(a00, a11, -(d01 * d10));
     // |det| must not be tiny against the entries
@@ -557,35 +569,84 @@ __device__ __forceinline__ void write_u_slices(const double* U, int w, unsigned 
 }
 
 // Dynamic shared memory needed by window_body: U, the packed window, the
-// transforms and swap lists of two steps, block-start and selection flags.
+// transforms and swap lists of two steps, selection flags.
 constexpr size_t kWindowSmem = sizeof(double) * ((size_t)WMAX * WMAX +
                                                  (size_t)((WMAX * (WMAX + 3)) / 2) +
                                                  (size_t)2 * MAXSW * 16) +
-                               sizeof(int) * 2 * 3 * MAXSW + 2 * WMAX;
+                               sizeof(int) * 2 * MAXSW + WMAX;
 // A wide window task keeps only the transforms, swap lists and flags here.
 constexpr size_t kWindowSmemWide = sizeof(double) * (size_t)2 * (WMAX_WIDE / 2) * 16 +
-                                   sizeof(int) * 2 * 3 * (WMAX_WIDE / 2) + 2 * WMAX_WIDE;
+                                   sizeof(int) * 2 * (WMAX_WIDE / 2) + WMAX_WIDE;
 
-// How a step's slot keeps its transformation Z (swk[slot] = k, plus Z_MATRIX
-// where the full transform computed it; swp[slot] tells 1|2 from 2|1):
+// A swap of a step: its slot's descriptor holds j (first row), k (rows), the
+// size p of the block above (0: a standardization rotation) and whether the
+// full transform computed it (Z_MATRIX).  A rejected swap has k = 0.  Slots
+// are numbered by size, k = 4 first, then k = 3, then k = 2.
+constexpr int Z_MATRIX = 16;
+__device__ __forceinline__ int sw_desc(int j, int kk, int p) { return j | (kk << 16) | (p << 24); }
+__device__ __forceinline__ int sw_j(int d) { return d & 0xffff; }
+__device__ __forceinline__ int sw_kk(int d) { return (d >> 16) & 0xff; }
+__device__ __forceinline__ int sw_p(int d) { return d >> 24; }
+
+// The slot's transformation Z (x <- x Z for a row x of K values, Z^T x for a
+// column):
 //   k = 2: Z = [[c, -s], [s, c]] as (c, s);
 //   k = 3: one reflector (w0, w1, f), in reversed index order for 1|2;
 //   k = 4: two reflectors (w0, w1, f) on 0..2 and (u0, u1, f') on 1..3;
 //   Z_MATRIX: the k x k matrix, column-major with leading dimension 4.
-// The reflectors take 6 and 12 FP64 instructions per row where the matrices
-// take 9 and 16.
-constexpr int Z_MATRIX = 16;
-
-// x <- x Z for one row x of K values (or Z^T x for a column).
+// The reflectors take 6 and 12 FP64 instructions where the matrices take 9
+// and 16.
+//
+// One item of a step's products: K values of the packed window or of U at a,
+// a + o1, a + o2, a + o3 and the slot's Z (reversed for a flipped reflector).
+struct Item {
+    double* a;
+    const double* z;
+    int o1, o2, o3;
+    bool ok, matrix;
+};
+// st, inc: the second value is st after the first, the step then grows by inc.
 template <int K>
-__device__ __forceinline__ void apply_z(const double* __restrict__ Z, bool matrix, double* x) {
+__device__ __forceinline__ Item make_item(double* a, int st, int inc, int d, const double* z, bool ok) {
+    Item t;
+    t.matrix = K > 2 && (sw_kk(d) & Z_MATRIX);
+    t.ok = ok && sw_kk(d) != 0;
+    t.a = a;
+    t.o1 = st;
+    t.o2 = 2 * st + inc;
+    t.o3 = 3 * (st + inc);
+    if (K == 3 && sw_p(d) == 1 && !t.matrix) {
+        t.a = a + t.o2;
+        t.o1 = -(st + inc);
+        t.o2 = -t.o2;
+    }
+    t.z = z;
+    return t;
+}
+template <int K>
+__device__ __forceinline__ void item_load(const Item& t, double* x) {
+    x[0] = t.a[0];
+    x[1] = t.a[t.o1];
+    if constexpr (K > 2) x[2] = t.a[t.o2];
+    if constexpr (K > 3) x[3] = t.a[t.o3];
+}
+template <int K>
+__device__ __forceinline__ void item_store(const Item& t, const double* x) {
+    t.a[0] = x[0];
+    t.a[t.o1] = x[1];
+    if constexpr (K > 2) t.a[t.o2] = x[2];
+    if constexpr (K > 3) t.a[t.o3] = x[3];
+}
+template <int K, bool MAT>
+__device__ __forceinline__ void item_apply(const Item& t, double* x) {
+    const double* Z = t.z;
     if constexpr (K == 2) {
         const double c = Z[0], s = Z[1];
         const double y = fma(s, x[1], c * x[0]);
         x[1] = fma(c, x[1], -(s * x[0]));
         x[0] = y;
     } else {
-        if (matrix) {
+        if (MAT && t.matrix) {
             double y[K];
 #pragma unroll
             for (int c = 0; c < K; ++c) {
@@ -602,42 +663,38 @@ __device__ __forceinline__ void apply_z(const double* __restrict__ Z, bool matri
         }
     }
 }
-
-// The slot's transformation on K values x0[0], x0[stride(1)], ...: rows
-// [j, j + K) of a column of the packed window (left), columns [j, j + K) of a
-// row of it or of U (right).  at(i) is the address of the i-th value.
-template <int K, typename At>
-__device__ __forceinline__ void apply_slot(const double* __restrict__ Z, int kk, int p, At at) {
-    const bool matrix = K > 2 && (kk & Z_MATRIX);
-    const bool flip = K == 3 && p == 1 && !matrix;
+// One item per lane, or two whose instructions interleave: an FP64 result is
+// 64 cycles away, and three product warps per sub-partition with one chain
+// each leave its pipe idle half of the time.  All lanes of the warp call.
+template <int K>
+__device__ __forceinline__ void item_run(const Item& t) {
+    if (!t.ok) return;
     double x[K];
+    item_load<K>(t, x);
+    item_apply<K, true>(t, x);
+    item_store<K>(t, x);
+}
+template <int K>
+__device__ __forceinline__ void item_run2(const Item& t, const Item& v) {
+    if (!__any_sync(0xffffffffu, v.ok) ||
+        (K > 2 && __any_sync(0xffffffffu, (t.ok && t.matrix) || (v.ok && v.matrix)))) {
+        item_run<K>(t);
+        item_run<K>(v);
+        return;
+    }
+    double x[K], y[K];
 #pragma unroll
-    for (int i = 0; i < K; ++i) x[i] = *at(K == 3 && flip ? K - 1 - i : i);
-    apply_z<K>(Z, matrix, x);
-#pragma unroll
-    for (int i = 0; i < K; ++i) *at(K == 3 && flip ? K - 1 - i : i) = x[i];
-}
-template <int K>
-__device__ __forceinline__ void left_col(double* __restrict__ Sp, int j, int c,
-                                         const double* __restrict__ Z, int kk, int p) {
-    double* x = Sp + poff(c) + j;
-    apply_slot<K>(Z, kk, p, [&](int i) { return x + i; });
-}
-template <int K>
-__device__ __forceinline__ void right_row(double* __restrict__ Sp, int j, int r,
-                                          const double* __restrict__ Z, int kk, int p) {
-    apply_slot<K>(Z, kk, p, [&](int i) { return Sp + poff(j + i) + r; });
-}
-template <int K>
-__device__ __forceinline__ void right_u_row(double* __restrict__ U, int w, int j, int r,
-                                            const double* __restrict__ Z, int kk, int p) {
-    double* x = U + j * w + r;
-    apply_slot<K>(Z, kk, p, [&](int i) { return x + i * w; });
+    for (int i = 0; i < K; ++i) x[i] = y[i] = 0.0;
+    if (t.ok) item_load<K>(t, x);
+    if (v.ok) item_load<K>(v, y);
+    item_apply<K, false>(t, x);
+    item_apply<K, false>(v, y);
+    if (t.ok) item_store<K>(t, x);
+    if (v.ok) item_store<K>(v, y);
 }
 
-// Last i in [0, cnt) with pre[i] <= it (pre is nondecreasing, pre[0] = 0).
-__device__ __forceinline__ int prefix_slot(const int* pre, int cnt, int it) {
-    int lo = 0, hi = cnt - 1;
+// Last i in [lo, hi] with pre[i] <= it (pre is nondecreasing, pre[lo] <= it).
+__device__ __forceinline__ int prefix_slot(const int* pre, int lo, int hi, int it) {
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (pre[mid] <= it) lo = mid; else hi = mid - 1;
@@ -709,16 +766,14 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
     double* U = WIDE ? Ug : reinterpret_cast<double*>(smem_raw);        // w*w
     double* Sp = WIDE ? gsp : U + WM * WM;                               // packed window
     double* Zbuf = WIDE ? reinterpret_cast<double*>(smem_raw) : Sp + poff(WM);  // [2][MSW * 16]
-    int* swbuf = reinterpret_cast<int*>(Zbuf + 2 * MSW * 16);  // [2][3][MSW]: j, k, p
-    uint8_t* bst = reinterpret_cast<uint8_t*>(swbuf + 2 * 3 * MSW);
-    uint8_t* sel = bst + WM;
-    __shared__ int nsw, nrej, nacc;
+    int* swbuf = reinterpret_cast<int*>(Zbuf + 2 * MSW * 16);  // [2][MSW]: descriptors
+    uint8_t* sel = reinterpret_cast<uint8_t*>(swbuf + 2 * MSW);
+    __shared__ int nsw[2], nrej, nacc;  // swaps of a step, by parity; rejected, accepted
     unsigned long long wflops = 0;   // per thread (phase D), summed at the end
-    __shared__ int tcnt2[2][3];
-    __shared__ int tlist2[2][3][MSW];     // slots per type (T_11, T_3, T_22: k = 2, 3, 4)
-    __shared__ int kpre_l2[2][3][MSW + 1];  // prefix sums of the far left-apply columns
-    __shared__ int kpre_s2[2][3][MSW + 1];  // prefix sums of the far right-apply rows of S
-    __shared__ int kpre_u2[2][3][MSW + 1];  // prefix sums of the right-apply rows of U
+    __shared__ int tcnt2[2][3];         // swaps per type (T_11, T_3, T_22: k = 2, 3, 4)
+    // prefix sums over the slots: far left-apply columns, far right-apply
+    // rows of S, right-apply rows of U
+    __shared__ int kpre_l2[2][MSW + 1], kpre_s2[2][MSW + 1], kpre_u2[2][MSW + 1];
     // Rows [urlo[c], urhi[c]] hold every nonzero of column c of U: U starts as
     // I and a swap on columns [j, j+k) mixes only those columns, so the rows
     // outside the union of their ranges stay exactly zero and are skipped.
@@ -766,126 +821,170 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
     if (tid == 0 && wall_top) sel[0] = SEL_WALL;
     if (tid == 0 && wall_bot) sel[w - 1] = SEL_WALL;
 
-    // --- phase A1 of the step of parity pi (integer work only): every
-    // selected block whose upper neighbour is an unselected block swaps with
-    // it.  In the final pass, the 2x2 blocks whose standard form has to be
-    // restored are listed instead (the fast swap paths leave it to this pass).
-    auto list_swaps = [&](int pi, bool fin) {
-        int* swj = swbuf + pi * 3 * MSW;
-        int* swk = swj + MSW;
-        int* swp = swk + MSW;
-        int (*tlist)[MSW] = tlist2[pi];
-        int* tcnt = tcnt2[pi];
-        if (!fin) {
-            for (int t = tid; t < w; t += nth) {
-                if (t == 0 || !bst[t] || sel[t] != SEL_YES) continue;
-                int ja = bst[t - 1] ? t - 1 : t - 2;
-                if (sel[ja] != SEL_NO) continue;
-                int p = t - ja;
-                int q = (t + 1 < w && !bst[t + 1]) ? 2 : 1;
-                int slot = atomicAdd(&nsw, 1);
-                swj[slot] = ja;
-                swk[slot] = p + q;
-                swp[slot] = p;
-                int ty = (p + q == 2) ? T_11 : (p + q == 3 ? T_3 : T_22);
-                tlist[ty][atomicAdd(&tcnt[ty], 1)] = slot;
+    // --- control of a step boundary, by one transform warp while the product
+    // warps start on the critical products (integer work on bit masks of the
+    // window's positions; with all warps and block barriers between its parts
+    // it took 3.4K cycles of a step's 24K).
+    //
+    // phase D of the step of parity pp with nsq swaps: move the selection
+    // flags with the blocks and widen the U row ranges of the columns each
+    // accepted transform mixed.
+    auto phase_d = [&](int pp, int nsq) {
+        const int* desc = swbuf + pp * MSW;
+        for (int sw = lane; sw < nsq; sw += 32) {
+            const int d = desc[sw], j = sw_j(d), p = sw_p(d), k = sw_kk(d) & (Z_MATRIX - 1);
+            if (k == 0) {
+                sel[j + p] = SEL_STUCK;  // the selected block
+                continue;
             }
-        } else {
-            for (int t = tid; t + 1 < w; t += nth) {
-                if (!bst[t] || bst[t + 1]) continue;  // 2x2 block at t
-                double m00 = Sp[poff(t) + t], m10 = Sp[poff(t) + t + 1];
-                double m01 = Sp[poff(t + 1) + t], m11 = Sp[poff(t + 1) + t + 1];
-                if (m00 == m11 && m01 * m10 < 0.0) continue;  // already standard
-                int slot = atomicAdd(&nsw, 1);
-                swj[slot] = t;
-                swk[slot] = 2;
-                swp[slot] = -1;   // marks a standardization rotation
-                tlist[T_11][atomicAdd(&tcnt[T_11], 1)] = slot;
+            const int lo = slo2[pp][sw], hi = shi2[pp][sw];
+            // in-window flops of this accepted transform: k x k applied to
+            // w - j - k columns (left) and j rows of S + its U rows (right)
+            wflops += 2ull * k * k * (unsigned long long)((w - j - k) + j + (hi - lo + 1));
+            const int q = k - p;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (c < k) {
+                    urlo[j + c] = (short)lo;
+                    urhi[j + c] = (short)hi;
+                    if (p > 0) sel[j + c] = c < q ? SEL_YES : SEL_NO;  // (0: blocks do not move)
+                }
+        }
+        __syncwarp();
+    };
+    // phase A1 of the step of parity pi: every selected block whose upper
+    // neighbour is an unselected block swaps with it.  In the final pass, the
+    // 2x2 blocks whose standard form has to be restored are listed instead
+    // (the fast swap paths leave it to this pass).  Returns the number of
+    // swaps; bit t & 31 of word t >> 5 stands for position t.
+    constexpr int NWORD = WM / 32;
+    auto list_swaps = [&](int pi, bool fin) {
+        int* desc = swbuf + pi * MSW;
+        unsigned bs[NWORD], sw[NWORD];     // block starts, swaps (by the selected block's start)
+        unsigned one[NWORD], two[NWORD];   // the block above is 1x1; a 2x2 block from here on
+        unsigned yes[NWORD], no[NWORD];    // selected, unselected
+        unsigned carry = 0;                // the word before ends in a stuck position
+#pragma unroll
+        for (int i = 0; i < NWORD; ++i) {
+            bs[i] = yes[i] = no[i] = 0u;
+            if (32 * i < w) {
+                const int t = 32 * i + lane;
+                const bool in = t < w;
+                const bool start = in && (t == 0 || is_zero(Sp[poff(t - 1) + t]));
+                const int f = in ? sel[t] : SEL_WALL;
+                bs[i] = __ballot_sync(0xffffffffu, start);
+                yes[i] = __ballot_sync(0xffffffffu, f == SEL_YES);
+                no[i] = __ballot_sync(0xffffffffu, f == SEL_NO);
+                // a stuck 2x2 block is flagged on both of its rows
+                const unsigned st = __ballot_sync(0xffffffffu, f == SEL_STUCK);
+                const unsigned both = ((st << 1) | carry) & ~bs[i];
+                if (both) {
+                    if (in && ((both >> lane) & 1u)) sel[t] = SEL_STUCK;
+                    yes[i] &= ~both;
+                    no[i] &= ~both;
+                }
+                carry = (st | both) >> 31;
             }
         }
+        int n4 = 0, n3 = 0, n2 = 0;
+#pragma unroll
+        for (int i = 0; i < NWORD; ++i) {
+            sw[i] = one[i] = two[i] = 0u;
+            if (32 * i < w) {
+                const unsigned bp = i ? bs[i > 0 ? i - 1 : 0] : 0u, np = i ? no[i > 0 ? i - 1 : 0] : 0u;
+                const unsigned bn = i + 1 < NWORD ? bs[i + 1 < NWORD ? i + 1 : i] : 0u;
+                const int left = w - 32 * i;  // positions from this word on
+                const unsigned more = left > 32 ? ~0u : (1u << (left - 1)) - 1u;  // t + 1 < w
+                one[i] = (bs[i] << 1) | (bp >> 31);
+                two[i] = ~((bs[i] >> 1) | (bn << 31)) & more;
+                if (!fin) {
+                    const unsigned nabove = (one[i] & ((no[i] << 1) | (np >> 31))) |
+                                            (~one[i] & ((no[i] << 2) | (np >> 30)));
+                    sw[i] = bs[i] & yes[i] & nabove;
+                    if (i == 0) sw[i] &= ~1u;
+                    n4 += __popc(sw[i] & ~one[i] & two[i]);
+                    n3 += __popc(sw[i] & (one[i] ^ ~two[i]));
+                    n2 += __popc(sw[i] & one[i] & ~two[i]);
+                } else {
+                    bool stale = false;
+                    const int t = 32 * i + lane;
+                    if (((bs[i] & two[i]) >> lane) & 1u) {
+                        const double m00 = Sp[poff(t) + t], m10 = Sp[poff(t) + t + 1];
+                        const double m01 = Sp[poff(t + 1) + t], m11 = Sp[poff(t + 1) + t + 1];
+                        stale = !(m00 == m11 && m01 * m10 < 0.0);
+                    }
+                    sw[i] = __ballot_sync(0xffffffffu, stale);
+                    n2 += __popc(sw[i]);
+                }
+            }
+        }
+        int at4 = 0, at3 = n4, at2 = n4 + n3;
+        const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+        for (int i = 0; i < NWORD; ++i) {
+            if (32 * i < w) {
+                const unsigned m4 = fin ? 0u : sw[i] & ~one[i] & two[i];
+                const unsigned m3 = fin ? 0u : sw[i] & (one[i] ^ ~two[i]), m2 = sw[i] & ~(m4 | m3);
+                if ((sw[i] >> lane) & 1u) {
+                    const int t = 32 * i + lane;
+                    const int p = (one[i] >> lane) & 1u ? 1 : 2, q = (two[i] >> lane) & 1u ? 2 : 1;
+                    const int slot = (m4 >> lane) & 1u   ? at4 + __popc(m4 & below)
+                                     : (m3 >> lane) & 1u ? at3 + __popc(m3 & below)
+                                                         : at2 + __popc(m2 & below);
+                    desc[slot] = fin ? sw_desc(t, 2, 0) : sw_desc(t - p, p + q, p);
+                }
+                at4 += __popc(m4);
+                at3 += __popc(m3);
+                at2 += __popc(m2);
+            }
+        }
+        if (lane < 3) tcnt2[pi][lane] = lane == T_11 ? n2 : (lane == T_3 ? n3 : n4);
+        return n4 + n3 + n2;
     };
 
-    // Prefix sums of the product work of the step of parity pi, per k group,
-    // by one warp: far left columns, far right rows of S, right rows of U
+    // Prefix sums of the product work of the ns swaps of the step of parity
+    // pi, by one warp: far left columns, far right rows of S, right rows of U
     // (whose range per swap, from urlo/urhi, it also records).  All listed
     // swaps are counted; a rejected one is skipped when applied.
-    auto prefix_sums = [&](int pi) {
-        const int* swj = swbuf + pi * 3 * MSW;
-#pragma unroll 1
-        for (int g = 0; g < 3; ++g) {
-            const int k = g + 2, cnt = tcnt2[pi][g];
-            int runl = 0, runr = 0, runu = 0;
-            for (int base = 0; base < cnt; base += 32) {
-                const int i = base + lane;
-                int nl = 0, nr = 0, nu = 0;
-                if (i < cnt) {
-                    const int slot = tlist2[pi][g][i], j = swj[slot];
+    auto prefix_sums = [&](int pi, int ns) {
+        const int* desc = swbuf + pi * MSW;
+        int runl = 0, runr = 0, runu = 0;
+        for (int base = 0; base < ns; base += 32) {
+            const int i = base + lane;
+            int nl = 0, nr = 0, nu = 0;
+            if (i < ns) {
+                // (a swap rejected by now has k = 0: no items)
+                const int d = desc[i], j = sw_j(d), k = sw_kk(d) & (Z_MATRIX - 1);
+                if (k > 0) {
                     int lo = urlo[j], hi = urhi[j];
                     for (int c = 1; c < k; ++c) {
                         lo = min(lo, (int)urlo[j + c]);
                         hi = max(hi, (int)urhi[j + c]);
                     }
-                    slo2[pi][slot] = (short)lo;
-                    shi2[pi][slot] = (short)hi;
+                    slo2[pi][i] = (short)lo;
+                    shi2[pi][i] = (short)hi;
                     nl = max(0, w - j - CRIT_L);
                     nr = max(0, j + k - CRIT_R);
                     nu = hi - lo + 1;
                 }
-                int il = nl, ir = nr, iu = nu;
-                for (int o = 1; o < 32; o <<= 1) {
-                    int a = __shfl_up_sync(0xffffffffu, il, o);
-                    int b2 = __shfl_up_sync(0xffffffffu, ir, o);
-                    int c2 = __shfl_up_sync(0xffffffffu, iu, o);
-                    if (lane >= o) { il += a; ir += b2; iu += c2; }
-                }
-                if (i < cnt) {
-                    kpre_l2[pi][g][i + 1] = runl + il;
-                    kpre_s2[pi][g][i + 1] = runr + ir;
-                    kpre_u2[pi][g][i + 1] = runu + iu;
-                }
-                runl += __shfl_sync(0xffffffffu, il, 31);
-                runr += __shfl_sync(0xffffffffu, ir, 31);
-                runu += __shfl_sync(0xffffffffu, iu, 31);
             }
-            if (lane == 0) {
-                kpre_l2[pi][g][0] = 0;
-                kpre_s2[pi][g][0] = 0;
-                kpre_u2[pi][g][0] = 0;
+            int il = nl, ir = nr, iu = nu;
+            for (int o = 1; o < 32; o <<= 1) {
+                int a = __shfl_up_sync(0xffffffffu, il, o);
+                int b2 = __shfl_up_sync(0xffffffffu, ir, o);
+                int c2 = __shfl_up_sync(0xffffffffu, iu, o);
+                if (lane >= o) { il += a; ir += b2; iu += c2; }
             }
+            if (i < ns) {
+                kpre_l2[pi][i + 1] = runl + il;
+                kpre_s2[pi][i + 1] = runr + ir;
+                kpre_u2[pi][i + 1] = runu + iu;
+            }
+            runl += __shfl_sync(0xffffffffu, il, 31);
+            runr += __shfl_sync(0xffffffffu, ir, 31);
+            runu += __shfl_sync(0xffffffffu, iu, 31);
         }
-    };
-
-    // --- phase D of the step of parity pp with nsq swaps: move the
-    // selection flags with the blocks; widen the U row ranges of the columns
-    // each accepted transform mixed; a stuck 2x2 block is flagged on both of
-    // its rows.  Needs the step's transforms only (not its products).
-    auto phase_d = [&](int pp, int nsq) {
-        const int* swj = swbuf + pp * 3 * MSW;
-        const int* swk = swj + MSW;
-        const int* swp = swk + MSW;
-        for (int sw = tid; sw < nsq; sw += nth) {
-            int j = swj[sw], k = swk[sw];
-            if (k == 0) {
-                sel[swp[sw]] = SEL_STUCK;
-                continue;
-            }
-            k &= Z_MATRIX - 1;
-            // in-window flops of this accepted transform: k x k applied to
-            // w - j - k columns (left) and j rows of S + its U rows (right)
-            wflops += 2ull * k * k *
-                      (unsigned long long)((w - j - k) + j + (shi2[pp][sw] - slo2[pp][sw] + 1));
-            for (int c = 0; c < k; ++c) {
-                urlo[j + c] = slo2[pp][sw];
-                urhi[j + c] = shi2[pp][sw];
-            }
-            int p = swp[sw], q = k - p;
-            if (p < 0) continue;   // standardization: blocks do not move
-            for (int i = 0; i < q; ++i) sel[j + i] = SEL_YES;
-            for (int i = q; i < k; ++i) sel[j + i] = SEL_NO;
-        }
-        __syncthreads();
-        for (int t = tid; t + 1 < w; t += nth)
-            if (sel[t] == SEL_STUCK && Sp[poff(t) + t + 1] != 0.0) sel[t + 1] = SEL_STUCK;
+        if (lane == 0) kpre_l2[pi][0] = kpre_s2[pi][0] = kpre_u2[pi][0] = 0;
     };
 
     // --- phase A2 of the step of parity pi, by the transform warps (warps
@@ -895,16 +994,13 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
     // rotations, dealt out in this order (the longest chains first).
     auto transforms = [&](int pi) {
         double* Zs = Zbuf + pi * MSW * 16;
-        int* swj = swbuf + pi * 3 * MSW;
-        int* swk = swj + MSW;
-        int* swp = swk + MSW;
-        const int (*tlist)[MSW] = tlist2[pi];
+        int* desc = swbuf + pi * MSW;
         const int* tcnt = tcnt2[pi];
         const int n22 = (tcnt[T_22] + 1) >> 1, n3 = (tcnt[T_3] + 7) >> 3;
         const int nunits = n22 + n3 + ((tcnt[T_11] + 31) >> 5);
         // the full transform of a swap, by one lane
         auto full = [&](int slot) {
-            const int ja = swj[slot], p = swp[slot], k = swk[slot];
+            const int ja = sw_j(desc[slot]), p = sw_p(desc[slot]), k = sw_kk(desc[slot]);
             double D[16], Zl[16], Dn[16];
             for (int cc = 0; cc < k; ++cc)
                 for (int rr = 0; rr < k; ++rr)
@@ -914,22 +1010,20 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                     for (int rr = 0; rr <= min(cc + 1, k - 1); ++rr)
                         Sp[poff(ja + cc) + ja + rr] = Dn[cc * 4 + rr];
                 for (int e = 0; e < 16; ++e) Zs[slot * 16 + e] = Zl[e];
-                swk[slot] = k | Z_MATRIX;
+                desc[slot] = sw_desc(ja, k | Z_MATRIX, p);
                 atomicAdd(&nacc, 1);
             } else {
-                swk[slot] = 0;
-                swp[slot] = ja + p;   // the stuck (selected) block
+                desc[slot] = sw_desc(ja, 0, p);
                 atomicAdd(&nrej, 1);
             }
         };
         for (int u = warp; u < nunits; u += NTW) {
             if (u < n22) {
                 // two 2|2 swaps, one per half-warp
-                const int h = lane >> 4, l = lane & 15, i = 2 * u + h;
+                const int h = lane >> 4, l = lane & 15, slot = 2 * u + h;
                 const unsigned hmask = h ? 0xffff0000u : 0x0000ffffu;
-                if (i < tcnt[T_22]) {
-                    const int slot = tlist[T_22][i];
-                    const int ja = swj[slot];
+                if (slot < tcnt[T_22]) {
+                    const int ja = sw_j(desc[slot]);
                     double z[6], dnrc = 0.0;
                     const bool ok = swap22_halfwarp(Sp, ja, l, hmask, h * 16, strong != 0, z, &dnrc);
                     const int r = l & 3, c = l >> 2;
@@ -949,9 +1043,9 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                 // eight k = 3 swaps, one per quad of lanes
                 const int q = lane & 3, i = 8 * (u - n22) + (lane >> 2);
                 const bool act = i < tcnt[T_3];
-                const int slot = tlist[T_3][act ? i : tcnt[T_3] - 1];
-                const int ja = swj[slot];
-                const bool flip = swp[slot] == 1;
+                const int slot = tcnt[T_22] + (act ? i : tcnt[T_3] - 1);
+                const int ja = sw_j(desc[slot]);
+                const bool flip = sw_p(desc[slot]) == 1;
                 double z[3], dn[3];
                 const bool ok = swap3_quad(Sp, ja, flip, q, lane & ~3, strong != 0, z, dn);
                 __syncwarp();
@@ -977,12 +1071,12 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                 // 32 rotations
                 const int i = 32 * (u - n22 - n3) + lane;
                 if (i < tcnt[T_11]) {
-                    const int slot = tlist[T_11][i];
-                    const int ja = swj[slot], p = swp[slot];
+                    const int slot = tcnt[T_22] + tcnt[T_3] + i;
+                    const int ja = sw_j(desc[slot]), p = sw_p(desc[slot]);
                     double* Z = &Zs[slot * 16];
                     double* c0 = Sp + poff(ja) + ja;
                     double* c1 = Sp + poff(ja + 1) + ja;
-                    if (p < 0) {
+                    if (p == 0) {
                         // restore the standard form of the 2x2 block at ja
                         double m[16];
                         m[0] = c0[0];
@@ -1022,177 +1116,145 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
     // warps may start), far left items, far right items of S and the right
     // items of U.  Within each part the items are grouped by k so that the
     // lanes of a warp run the same k, and whole warps claim 32 items at a
-    // time (claim counters pclaim): an FP64 instruction holds its
+    // time (one claim counter per part): an FP64 instruction holds its
     // sub-partition's pipe for the same time with 1 or 32 lanes, and the
     // transform warps load some sub-partitions' pipes more than others, so
     // the warps of the less loaded sub-partitions take more items.
     // has = the step had swaps; the barriers run either way.
-    __shared__ int pclaim[5][3];
+    __shared__ int pclaim[2][4];  // by the parity of the step applied
     auto products = [&](int pp, bool has) {
         const double* Zs = Zbuf + pp * MSW * 16;
-        const int* swj = swbuf + pp * 3 * MSW;
-        const int* swk = swj + MSW;
-        const int* swp = swk + MSW;
-        const int (*tlist)[MSW] = tlist2[pp];
-        const int* tcnt = tcnt2[pp];
+        const int* desc = swbuf + pp * MSW;
+        const int m4 = tcnt2[pp][T_22], m3 = tcnt2[pp][T_3], m2 = tcnt2[pp][T_11];
         constexpr int NCL = CRIT_L - 2, NCR = CRIT_R - 2;  // item slots per swap
-        // next item of part `ph`, group g for this lane (or >= total: done)
-        auto claim = [&](int ph, int g) {
-            int base = 0;
-            if (lane == 0) base = atomicAdd(&pclaim[ph][g], 32);
-            return __shfl_sync(0xffffffffu, base, 0) + lane;
+        constexpr int NPW = WIN_THREADS / 32 - NTW;        // product warps
+        // The items of part `ph` (t4, t3, t2 of them per size), by chunks of
+        // one size, those with the most work per item first: PER items per
+        // lane (one for k = 4).  The first chunk of a warp is its own; the
+        // claim of the next one is under way while it works.
+        auto part = [&](auto PER, int ph, int t4, int t3, int t2, auto&& item) {
+            constexpr int per = decltype(PER)::value;
+            const int c4 = (t4 + 31) / 32, c3 = c4 + (t3 + 32 * per - 1) / (32 * per);
+            const int n = c3 + (t2 + 32 * per - 1) / (32 * per);
+            auto chunk = [&](auto K, int base, int t) {
+                constexpr int k = decltype(K)::value;
+                const int it = base + lane;
+                if constexpr (k == 4 || per == 1)
+                    item_run<k>(item(K, min(it, t - 1), it < t));
+                else
+                    item_run2<k>(item(K, min(it, t - 1), it < t), item(K, min(it + 32, t - 1), it + 32 < t));
+            };
+            for (int c = warp - NTW; c < n;) {
+                int nx = 0;
+                if (n > NPW && lane == 0) nx = atomicAdd(&pclaim[pp][ph], 1);
+                if (c < c4)
+                    chunk(std::integral_constant<int, 4>{}, 32 * c, t4);
+                else if (c < c3)
+                    chunk(std::integral_constant<int, 3>{}, 32 * per * (c - c4), t3);
+                else
+                    chunk(std::integral_constant<int, 2>{}, 32 * per * (c - c3), t2);
+                if (n <= NPW) break;
+                c = NPW + __shfl_sync(0xffffffffu, nx, 0);
+            }
         };
-        if (has) {
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const int k = g + 2, total = tcnt[g] * NCL;
-                for (int it = claim(0, g); it - lane < total; it = claim(0, g)) {
-                    if (it >= total) continue;
-                    const int slot = tlist[g][it / NCL];
-                    const int kk = swk[slot];
-                    if (kk == 0) continue;  // rejected
-                    const int j = swj[slot], c = j + k + it % NCL;
-                    if (c >= min(w, j + CRIT_L)) continue;
-                    const double* Z = Zs + slot * 16;
-                    if (g == 0) left_col<2>(Sp, j, c, Z, kk, swp[slot]);
-                    else if (g == 1) left_col<3>(Sp, j, c, Z, kk, swp[slot]);
-                    else left_col<4>(Sp, j, c, Z, kk, swp[slot]);
-                }
-            }
-        }
+        // slots of size k: first one and their number
+        auto first = [&](int k) { return k == 4 ? 0 : (k == 3 ? m4 : m4 + m3); };
+        auto many = [&](int k) { return k == 4 ? m4 : (k == 3 ? m3 : m2); };
+        constexpr std::integral_constant<int, 1> PER1{};
+        constexpr std::integral_constant<int, 2> PER2{};
+        if (has)
+            part(PER1, 0, m4 * NCL, m3 * NCL, m2 * NCL, [&](auto K, int it, bool ok) {
+                constexpr int k = decltype(K)::value;
+                const int slot = first(k) + it / NCL, d = desc[slot], j = sw_j(d), c = j + k + it % NCL;
+                return make_item<k>(Sp + poff(c) + j, 1, 0, d, Zs + slot * 16, ok && c < min(w, j + CRIT_L));
+            });
         bar_products();
-        if (has) {
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const int k = g + 2, total = tcnt[g] * NCR;
-                for (int it = claim(1, g); it - lane < total; it = claim(1, g)) {
-                    if (it >= total) continue;
-                    const int slot = tlist[g][it / NCR];
-                    const int kk = swk[slot];
-                    if (kk == 0) continue;
-                    const int j = swj[slot], r = j - 1 - it % NCR;
-                    if (r < max(0, j + k - CRIT_R)) continue;
-                    const double* Z = Zs + slot * 16;
-                    if (g == 0) right_row<2>(Sp, j, r, Z, kk, swp[slot]);
-                    else if (g == 1) right_row<3>(Sp, j, r, Z, kk, swp[slot]);
-                    else right_row<4>(Sp, j, r, Z, kk, swp[slot]);
-                }
-            }
-        }
+        if (has)
+            part(PER1, 1, m4 * NCR, m3 * NCR, m2 * NCR, [&](auto K, int it, bool ok) {
+                constexpr int k = decltype(K)::value;
+                const int slot = first(k) + it / NCR, d = desc[slot], j = sw_j(d), r = j - 1 - it % NCR;
+                return make_item<k>(Sp + poff(j) + r, j + 2, 1, d, Zs + slot * 16,
+                                    ok && r >= max(0, j + k - CRIT_R));
+            });
         __threadfence_block();
         bar_crit_arrive();
-        if (has) {
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const int cnt = tcnt[g];
-                const int* pre = kpre_l2[pp][g];
-                const int total = pre[cnt];
-                for (int it = claim(2, g); it - lane < total; it = claim(2, g)) {
-                    if (it >= total) continue;
-                    const int lo = prefix_slot(pre, cnt, it);
-                    const int slot = tlist[g][lo];
-                    const int kk = swk[slot];
-                    if (kk == 0) continue;
-                    const int j = swj[slot], c = j + CRIT_L + (it - pre[lo]);
-                    const double* Z = Zs + slot * 16;
-                    if (g == 0) left_col<2>(Sp, j, c, Z, kk, swp[slot]);
-                    else if (g == 1) left_col<3>(Sp, j, c, Z, kk, swp[slot]);
-                    else left_col<4>(Sp, j, c, Z, kk, swp[slot]);
-                }
-            }
-        }
+        const int* pl = kpre_l2[pp];
+        const int* ps = kpre_s2[pp];
+        const int* pu = kpre_u2[pp];
+        if (has)
+            part(PER2, 2, pl[m4], pl[m4 + m3] - pl[m4], pl[m4 + m3 + m2] - pl[m4 + m3],
+                 [&](auto K, int it, bool ok) {
+                     constexpr int k = decltype(K)::value;
+                     const int f = first(k);
+                     it += pl[f];
+                     const int slot = prefix_slot(pl, f, f + many(k) - 1, it), d = desc[slot], j = sw_j(d);
+                     return make_item<k>(Sp + poff(j + CRIT_L + (it - pl[slot])) + j, 1, 0, d, Zs + slot * 16,
+                                         ok);
+                 });
         bar_products();
         if (has) {
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const int cnt = tcnt[g];
-                const int* pre = kpre_s2[pp][g];
-                const int total = pre[cnt];
-                for (int it = claim(3, g); it - lane < total; it = claim(3, g)) {
-                    if (it >= total) continue;
-                    const int lo = prefix_slot(pre, cnt, it);
-                    const int slot = tlist[g][lo];
-                    const int kk = swk[slot];
-                    if (kk == 0) continue;
-                    const int j = swj[slot], r = it - pre[lo];
-                    const double* Z = Zs + slot * 16;
-                    if (g == 0) right_row<2>(Sp, j, r, Z, kk, swp[slot]);
-                    else if (g == 1) right_row<3>(Sp, j, r, Z, kk, swp[slot]);
-                    else right_row<4>(Sp, j, r, Z, kk, swp[slot]);
-                }
-            }
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const int cnt = tcnt[g];
-                const int* pre = kpre_u2[pp][g];
-                const int total = pre[cnt];
-                for (int it = claim(4, g); it - lane < total; it = claim(4, g)) {
-                    if (it >= total) continue;
-                    const int lo = prefix_slot(pre, cnt, it);
-                    const int slot = tlist[g][lo];
-                    const int kk = swk[slot];
-                    if (kk == 0) continue;
-                    const int j = swj[slot], r = slo2[pp][slot] + (it - pre[lo]);
-                    const double* Z = Zs + slot * 16;
-                    if (g == 0) right_u_row<2>(U, w, j, r, Z, kk, swp[slot]);
-                    else if (g == 1) right_u_row<3>(U, w, j, r, Z, kk, swp[slot]);
-                    else right_u_row<4>(U, w, j, r, Z, kk, swp[slot]);
-                }
-            }
+            // far right rows of S, then the rows of U, of each size
+            const int s4 = ps[m4], s3 = ps[m4 + m3] - s4, s2 = ps[m4 + m3 + m2] - ps[m4 + m3];
+            part(PER2, 3, s4 + pu[m4], s3 + pu[m4 + m3] - pu[m4], s2 + pu[m4 + m3 + m2] - pu[m4 + m3],
+                 [&](auto K, int it, bool ok) {
+                     constexpr int k = decltype(K)::value;
+                     const int ns = k == 4 ? s4 : (k == 3 ? s3 : s2), f = first(k);
+                     const bool u = it >= ns;
+                     const int* pre = u ? pu : ps;
+                     it += pre[f] - (u ? ns : 0);
+                     const int slot = prefix_slot(pre, f, f + many(k) - 1, it), d = desc[slot], j = sw_j(d);
+                     it -= pre[slot];
+                     double* a = u ? U + j * w + slo2[pp][slot] + it : Sp + poff(j) + it;
+                     return make_item<k>(a, u ? w : j + 2, u ? 0 : 1, d, Zs + slot * 16, ok);
+                 });
         }
     };
 
-    // Step pipeline.  Iteration i: the selection flags of step i - 1 move
-    // (phase D), step i's swaps are listed (phase A1), then the product warps
-    // apply step i - 1 while the transform warps compute step i.  Every
+    // Step pipeline.  Iteration i: one warp moves the selection flags of step
+    // i - 1 (phase D) and lists step i's swaps (phase A1), then the product
+    // warps apply step i - 1 while the transform warps compute step i.  Every
     // accepted swap moves a selected block up and every rejected one retires
     // a block, so the steps end within w * w; the cap only guards against a
     // logic error (reported through the counters).
-    bool final_pass = false, overflow = false;
+    bool fin = false;  // the final pass (warp 0)
     int ns_prev = 0;
+    if (tid < 8) pclaim[tid >> 2][tid & 3] = 0;
+    __syncthreads();
     for (int iter = 0;; ++iter) {
         const int pi = iter & 1, pp = pi ^ 1;
-        if (ns_prev > 0) phase_d(pp, ns_prev);
-        __syncthreads();
-        if (abort_word && !final_pass && nrej > 0) {
-            // ABORT: the first rejection stops the reordering; this window
-            // only restores the standard form of its 2x2 blocks
-            final_pass = true;
-            if (tid == 0) atomicExch(abort_word, 1);
-        }
-        if (iter > 4 * WM * WM && !overflow) {
-            if (tid == 0) atomicAdd(&ctr->step_overflow, 1);
-            overflow = true;
-        }
-        for (int i = tid; i < w; i += nth) bst[i] = (i == 0) || (Sp[poff(i - 1) + i] == 0.0);
-        if (tid < 3) tcnt2[pi][tid] = 0;
-        if (tid < 15) pclaim[tid / 3][tid % 3] = 0;
-        if (tid == 0) nsw = 0;
-        __syncthreads();
-        if (!overflow) list_swaps(pi, final_pass);
-        __syncthreads();
-        int ns = nsw;
-        if (ns == 0 && !final_pass && !overflow) {
-            // after the last swap: the pass that restores standard forms
-            final_pass = true;
-            __syncthreads();
-            if (tid < 3) tcnt2[pi][tid] = 0;
-            if (tid == 0) nsw = 0;
-            __syncthreads();
-            list_swaps(pi, true);
-            __syncthreads();
-            ns = nsw;
-        }
         if (warp < NTW) {
-            if (warp == NTW - 1 && ns > 0) prefix_sums(pi);
+            if (warp == 0) {
+                if (ns_prev > 0) phase_d(pp, ns_prev);
+                if (abort_word && !fin && nrej > 0) {
+                    // ABORT: the first rejection stops the reordering; this
+                    // window only restores the standard form of its 2x2 blocks
+                    fin = true;
+                    if (lane == 0) atomicExch(abort_word, 1);
+                }
+                int ns = 0;
+                if (iter > 4 * WM * WM) {
+                    if (lane == 0) atomicAdd(&ctr->step_overflow, 1);
+                } else {
+                    ns = list_swaps(pi, fin);
+                    if (ns == 0 && !fin) {
+                        // after the last swap: the pass that restores standard forms
+                        fin = true;
+                        ns = list_swaps(pi, true);
+                    }
+                }
+                if (lane < 4) pclaim[pi][lane] = 0;
+                if (lane == 0) nsw[pi] = ns;
+            }
             bar_crit_wait();
+            const int ns = nsw[pi];
             if (ns > 0) transforms(pi);
+            if (warp == NTW - 1 && ns > 0) prefix_sums(pi, ns);
         } else {
             products(pp, ns_prev > 0);
         }
         __syncthreads();
-        ns_prev = ns;
-        if (ns == 0) break;
+        ns_prev = nsw[pi];
+        if (ns_prev == 0) break;
     }
     __shared__ unsigned long long wfl_sum;
     if (tid == 0) wfl_sum = 0;
