@@ -27,6 +27,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "seeded.cuh"
 
 #include <float.h>
 
@@ -57,17 +58,20 @@ __device__ __forceinline__ unsigned long long mag(double x) {
 // ---------------------------------------------------------------------------
 // Swap of one pair of adjacent blocks by an octet: 8 lanes of a warp.
 //
-// An FP64 instruction costs the same issue slot for 1 or 32 active lanes, so
-// the swap's arithmetic is spread over 8 lanes instead of running on one:
-//   - the Kronecker system (N = 2pq <= 8 unknowns): lane r owns row r;
-//     complete pivoting by an octet arg-max (integer compares on the bit
-//     patterns), row and column exchanges by shuffles, one division per
-//     elimination step; back substitution column by column;
+// An FP64 instruction holds its sub-partition's pipe for 64 cycles whatever
+// its active lanes, and the swap is one dependent chain; so the arithmetic is
+// spread over 8 lanes, and FP32 and the special function unit give the first
+// approximations:
+//   - the Kronecker system (N = 2pq <= 8 unknowns): lane r owns row r of an
+//     FP32 inverse, refined with FP64 residuals (gen_sylv_seeded);
 //   - the two QR factors: lanes 0-3 build column l of Qs, lanes 4-7 column
 //     l - 4 of Zs (each half from its own reflectors);
 //   - the 4 x 4 products, the tests and the rotations of T's new 2x2 blocks:
 //     lane l owns entries 2l, 2l + 1 (column l / 2) of each k x k result,
 //     exchanged through the slot's shared-memory scratch.
+// Measured (pair window tasks of w = 64, m = 32, median in the schedule of an
+// n = 2000 pair): 1.67 ms with the elimination, roots and divisions in FP64,
+// 1.01 ms so.
 // All loops have the same trip counts on the 8 lanes; shuffles and
 // __syncwarp name the octet's lanes only.
 // ---------------------------------------------------------------------------
@@ -85,73 +89,13 @@ __device__ __forceinline__ double pick8(const double (&v)[8], int i) {
     return r;
 }
 
-// Reflector (I - tau v v^T) on 4-vectors mapping x onto beta e_0, v[0] = 1;
-// tau = 0 when x is a multiple of e_0 already.
-__device__ __forceinline__ void house4(const double x[4], double v[4], double* tau) {
-    const double sigma = fma(x[1], x[1], fma(x[2], x[2], x[3] * x[3]));
-    v[0] = 1.0;
-    v[1] = x[1];
-    v[2] = x[2];
-    v[3] = x[3];
-    *tau = 0.0;
-    if (sigma != 0.0) {
-        const double nrm = sqrt(fma(x[0], x[0], sigma));
-        const double beta = x[0] >= 0.0 ? -nrm : nrm;
-        const double inv = 1.0 / (x[0] - beta);
-        v[1] *= inv;
-        v[2] *= inv;
-        v[3] *= inv;
-        *tau = (beta - x[0]) / beta;
-    }
-}
-
-// Returns true (on all 8 lanes) if the swap of the p x p block at ja with the
-// q x q block below it is accepted; sc (the slot's scratch) then holds Qs,
-// Zs and the new diagonal parts NA, NB.  l: lane in the octet; ob: lane of
-// the octet's lane 0 in the warp; om: the octet's lane mask.
-__device__ __forceinline__ bool gen_swap_octet(int p, int q, const double* __restrict__ Sp,
-                                               const double* __restrict__ Tp, int ja, bool strong,
-                                               int l, int ob, unsigned om, double* __restrict__ sc) {
-    const int k = p + q, pq = p * q, N = 2 * pq;
-    // own entries e = 2l, 2l+1: column c0 = l / 2, rows r0, r0 + 1
-    const int ec = l >> 1, er = (l & 1) * 2;
-    double pa = 0.0, pb = 0.0;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        const int r = er + t;
-        const bool in = ec < k && r < k && r <= ec + 1;
-        const double a = in ? Sp[gpoff(ja + ec) + ja + r] : 0.0;
-        const double b = in ? Tp[gpoff(ja + ec) + ja + r] : 0.0;
-        sc[SC_DA + ec * 4 + r] = a;
-        sc[SC_DB + ec * 4 + r] = b;
-        pa = fma(a, a, pa);
-        pb = fma(b, b, pb);
-    }
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-        pa += __shfl_xor_sync(om, pa, o);
-        pb += __shfl_xor_sync(om, pb, o);
-    }
-    const double tha = fmax(20.0 * DBL_EPSILON * sqrt(pa), DBL_MIN);
-    const double thb = fmax(20.0 * DBL_EPSILON * sqrt(pb), DBL_MIN);
-    __syncwarp(om);
-    const double* DA = sc + SC_DA;
-    const double* DB = sc + SC_DB;
-    if (k == 2 && DA[0] * DB[5] == DA[5] * DB[0]) {
-        // equal generalized eigenvalues: in order already (identity factors)
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const int e = 2 * l + t;
-            const double id = ((e & 3) == (e >> 2)) ? 1.0 : 0.0;
-            sc[SC_Q + e] = id;
-            sc[SC_Z + e] = id;
-            sc[SC_NA + e] = DA[e];
-            sc[SC_NB + e] = DB[e];
-        }
-        __syncwarp(om);
-        return true;
-    }
-
+// The elimination with complete pivoting in FP64, for the swaps whose
+// FP32-seeded solution does not converge (out of line: it is rare).  Returns
+// unknown l on lane l < N; *g is its scaling against overflow.
+static __device__ __noinline__ double gen_sylv_full(int p, int q, const double* __restrict__ DA,
+                                                    const double* __restrict__ DB, int l, int ob,
+                                                    unsigned om, double* gout) {
+    const int pq = p * q, N = 2 * pq;
     // --- Kronecker row l: unknowns [vec R; vec L], equations [first; second]
     double K[8], b = 0.0;
 #pragma unroll
@@ -254,53 +198,227 @@ __device__ __forceinline__ bool gen_swap_octet(int p, int q, const double* __res
         const double ys = __shfl_sync(om, y, ob + s);
         if (l < s) acc = fma(-pick8(K, s), ys, acc);
     }
-    // unknown perm[c] = y of lane c: gather R (lanes 0-3 need L, 4-7 need R)
-    double X[4] = {0.0, 0.0, 0.0, 0.0};
-    const bool zhalf = l >= 4;
+    // unknown perm[c] is the y of lane c
+    double v = 0.0;
     for (int c = 0; c < N; ++c) {
-        const double v = __shfl_sync(om, y, ob + c);
+        const double yc = __shfl_sync(om, y, ob + c);
         const int u = __shfl_sync(om, perm, ob + c);
-        const int want = zhalf ? (u < pq ? u : -1) : u - pq;   // R for Zs, L for Qs
-#pragma unroll
-        for (int t = 0; t < 4; ++t) X[t] = (want == t) ? v : X[t];
+        v = u == l ? yc : v;
     }
+    *gout = g;
+    return v;
+}
+
+// The same system solved by an FP32 inverse (Gauss-Jordan in place, rows on
+// lanes, partial pivoting without exchanging rows) and refined with FP64
+// residuals until a correction is at most 2^-36 of the solution (the
+// correction after it would be below 2^-53, see swap22_halfwarp in
+// window_body.cuh).  The equations of A and of B are scaled by the power of
+// two of the matrix's largest entry; ea, eb: those exponent fields.  Returns
+// unknown l on lane l < N, *good on all lanes.
+//
+// Five FP64 instructions a correction, two corrections as a rule; the
+// elimination in FP64 takes about 20 per unknown and a dependent division.
+__device__ __forceinline__ double gen_sylv_seeded(int p, int q, const double* __restrict__ DA,
+                                                  const double* __restrict__ DB, int l, int ob,
+                                                  unsigned om, int ea, int eb, bool* good) {
+    const int sp = p - 1, pq = p * q, N = 2 * pq;  // division by p is a shift
+    // row l: X11[i][:] R[:][cc] - L[i][:] X22[:][cc] = -X12[i][cc], X = A or B
+    const int eq = l >= pq, rem = l - (eq ? pq : 0), i = rem & sp, cc = rem >> sp;
+    const bool row = l < N;
+    const int eoff = (eq ? eb : ea) - 127;
+    double c0 = 0.0, c1 = 0.0, d0 = 0.0, d1 = 0.0, b = 0.0;
+    if (row) {
+        const double* D = eq ? DB : DA;
+        b = -D[(p + cc) * 4 + i];
+        c0 = D[i];
+        if (p == 2) c1 = D[4 + i];
+        d0 = D[(p + cc) * 4 + p];
+        if (q == 2) d1 = D[(p + cc) * 4 + p + 1];
+    }
+    const float fc0 = to_f32(c0, eoff), fc1 = to_f32(c1, eoff);
+    const float fd0 = to_f32(d0, eoff), fd1 = to_f32(d1, eoff);
+    float k[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const int u = c - pq;
+        k[c] = !row || c >= N ? (c == l ? 1.0f : 0.0f)
+               : c < pq       ? ((c >> sp) == cc ? ((c & sp) ? fc1 : fc0) : 0.0f)
+                              : ((u & sp) == i ? -((u >> sp) ? fd1 : fd0) : 0.0f);
+    }
+    unsigned piv = 0;  // 3 bits per column: the lane of its pivot
+    bool used = !row, singular = false;
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+        if (s < N) {
+            unsigned key = used ? 0u : ((__float_as_uint(k[s]) & 0x7ffffff8u) | (unsigned)l);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) key = max(key, __shfl_xor_sync(om, key, o));
+            const int pl = key & 7;
+            singular |= key < 8u;
+            piv |= (unsigned)pl << (3 * s);
+            const bool mine = l == pl;
+            const float rp = __fdividef(1.0f, __shfl_sync(om, k[s], ob + pl));
+            const float f = mine ? 0.0f : k[s];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c != s && c < N) {
+                    const float v = __shfl_sync(om, k[c], ob + pl) * rp;
+                    k[c] = mine ? v : fmaf(-f, v, k[c]);
+                }
+            k[s] = mine ? rp : -f * rp;
+            used = used || mine;
+        }
+    }
+    // unknown l (on lane l < N) for the right-hand side r of row l
+    auto solve = [&](float r) {
+        float x = 0.0f;
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+            if (s < N) x = fmaf(k[s], __shfl_sync(om, r, ob + (int)((piv >> (3 * s)) & 7u)), x);
+        x = __shfl_sync(om, x, ob + (int)((piv >> (3 * l)) & 7u));
+        return row ? x : 0.0f;
+    };
+    auto omax = [&](float v) {  // largest |v| of the octet, NaN above all
+        unsigned m = __float_as_uint(v) & 0x7fffffffu;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(om, m, o));
+        return __uint_as_float(m);
+    };
+    float x = solve(to_f32(b, eoff));
+    const float xmax = omax(x);
+    double y = from_f32(x);
+    const int r0 = ob + (row ? cc << sp : 0), l0 = ob + (row ? pq + i : 0);
+    *good = false;
+#pragma unroll 1
+    for (int it = 0; it < 6 && !singular; ++it) {
+        double res = fma(-c0, __shfl_sync(om, y, r0), b);
+        res = fma(d0, __shfl_sync(om, y, l0), res);
+        res = fma(-c1, __shfl_sync(om, y, r0 + sp), res);
+        res = fma(d1, __shfl_sync(om, y, q == 2 ? l0 + p : l0), res);
+        x = solve(to_f32(res, eoff));
+        const float dmax = omax(x);
+        y += from_f32(x);
+        if (!(dmax <= 0.25f * xmax)) break;  // also NaN: no convergence
+        if (it > 0 && dmax <= 1.4551915e-11f * xmax) { *good = xmax < 1e30f; break; }
+    }
+    return y;
+}
+
+// Reflector I - f w w^T on 4-vectors mapping (a0, a1, a2, a3) onto
+// -sign(a0) |a| e_0: w = (w0, a1, a2, a3), f = 2 / |w|^2 from the rounded w.
+// |a| is in the normal range: one of a1..a3 is 1 (or the solution's scaling).
+__device__ __forceinline__ void refl4(double a0, double a1, double a2, double a3, double* w0,
+                                      double* f) {
+    const double sg = fma(a1, a1, fma(a2, a2, a3 * a3));
+    const double d = fabs(a0) + sqrt64(fma(a0, a0, sg));
+    *w0 = nonneg(a0) ? d : -d;
+    *f = rcp64(half_of(fma(d, d, sg)));
+}
+
+// Returns true (on all 8 lanes) if the swap of the p x p block at ja with the
+// q x q block below it is accepted; sc (the slot's scratch) then holds Qs,
+// Zs and the new diagonal parts NA, NB.  l: lane in the octet; ob: lane of
+// the octet's lane 0 in the warp; om: the octet's lane mask.
+__device__ __forceinline__ bool gen_swap_octet(int p, int q, const double* __restrict__ Sp,
+                                               const double* __restrict__ Tp, int ja, bool strong,
+                                               int l, int ob, unsigned om, double* __restrict__ sc) {
+    const int k = p + q, pq = p * q;
+    // own entries e = 2l, 2l+1: column c0 = l / 2, rows r0, r0 + 1
+    const int ec = l >> 1, er = (l & 1) * 2;
+    const bool zhalf = l >= 4;
+    double pa = 0.0, pb = 0.0;
+    int ea = 0, eb = 0;  // largest exponent fields of A and B
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int r = er + t;
+        const bool in = ec < k && r < k && r <= ec + 1;
+        const double a = in ? Sp[gpoff(ja + ec) + ja + r] : 0.0;
+        const double b = in ? Tp[gpoff(ja + ec) + ja + r] : 0.0;
+        sc[SC_DA + ec * 4 + r] = a;
+        sc[SC_DB + ec * 4 + r] = b;
+        pa = fma(a, a, pa);
+        pb = fma(b, b, pb);
+        ea = max(ea, (__double2hiint(a) >> 20) & 0x7ff);
+        eb = max(eb, (__double2hiint(b) >> 20) & 0x7ff);
+    }
+    // sums over the octet: A's on lanes 0-3, B's on lanes 4-7
+    double ps = zhalf ? pb : pa;
+    ps += __shfl_xor_sync(om, zhalf ? pa : pb, 4);
+    ps += __shfl_xor_sync(om, ps, 1);
+    ps += __shfl_xor_sync(om, ps, 2);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        ea = max(ea, __shfl_xor_sync(om, ea, o));
+        eb = max(eb, __shfl_xor_sync(om, eb, o));
+    }
+    // thresholds max(20 eps ||.||_F, DBL_MIN) as bit patterns; a sum outside
+    // the normal range takes the plain square root
+    unsigned long long th;
+    {
+        const int e = (__double2hiint(ps) >> 20) & 0x7ff;
+        const double nf = e > 64 && e < 2047 ? sqrt64(ps) : sqrt(ps);
+        th = mag(20.0 * DBL_EPSILON * nf);
+        th = th > 0x0010000000000000ULL ? th : 0x0010000000000000ULL;
+    }
+    const unsigned long long tha = __shfl_sync(om, th, ob), thb = __shfl_sync(om, th, ob + 4);
+    __syncwarp(om);
+    const double* DA = sc + SC_DA;
+    const double* DB = sc + SC_DB;
+    if (k == 2 && DA[0] * DB[5] == DA[5] * DB[0]) {
+        // equal generalized eigenvalues: in order already (identity factors)
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int e = 2 * l + t;
+            const double id = ((e & 3) == (e >> 2)) ? 1.0 : 0.0;
+            sc[SC_Q + e] = id;
+            sc[SC_Z + e] = id;
+            sc[SC_NA + e] = DA[e];
+            sc[SC_NB + e] = DB[e];
+        }
+        __syncwarp(om);
+        return true;
+    }
+
+    // --- generalized Sylvester equation: unknowns [vec R; vec L] on lanes
+    double g = 1.0;
+    bool good;
+    double y = gen_sylv_seeded(p, q, DA, DB, l, ob, om, ea, eb, &good);
+    if (!good) y = gen_sylv_full(p, q, DA, DB, l, ob, om, &g);
     // --- QR factor: column (l & 3) of Qs (lanes 0-3, from [L; g I]) or of
     // Zs (lanes 4-7, from [R; g I]); H1 for column 0, H2 on rows 1..3
     {
-        double M0[4], M1[4];
+        double X[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            M0[i] = i < p ? X[i] : (i == p ? g : 0.0);
-            M1[i] = (q == 2) ? (i < p ? X[i + p] : (i == p + 1 ? g : 0.0)) : 0.0;
+        for (int t = 0; t < 4; ++t) {
+            const double v = __shfl_sync(om, y, ob + (t < pq ? (zhalf ? t : pq + t) : 0));
+            X[t] = t < pq ? v : 0.0;
         }
-        double v1[4], v2[4], t1, t2 = 0.0;
-        house4(M0, v1, &t1);
-        v2[0] = 1.0; v2[1] = v2[2] = v2[3] = 0.0;
+        // [X; g I]: columns (X0, X1, g, 0), (X2, X3, 0, g) for p = 2,
+        // (X0, g, 0, 0), (X1, 0, g, 0) for p = 1
+        const double a1 = p == 2 ? X[1] : g, a2 = p == 2 ? g : 0.0;
+        double w0, f1;
+        refl4(X[0], a1, a2, 0.0, &w0, &f1);
+        double u0 = 1.0, u1 = 0.0, u2 = 0.0, f2 = 0.0;
         if (q == 2) {
-            double d = 0.0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) d = fma(v1[i], M1[i], d);
-            d *= t1;
-            double x2[4];
-#pragma unroll
-            for (int i = 1; i < 4; ++i) x2[i - 1] = fma(-d, v1[i], M1[i]);
-            x2[3] = 0.0;
-            house4(x2, v2, &t2);
+            const double m0 = p == 2 ? X[2] : X[1], m1 = p == 2 ? X[3] : 0.0, m2 = p == 2 ? 0.0 : g;
+            const double d = fma(w0, m0, fma(a1, m1, a2 * m2)) * f1;
+            const double x1 = fma(-d, a1, m1);
+            u1 = fma(-d, a2, m2);
+            u2 = p == 2 ? g : 0.0;
+            refl4(x1, u1, u2, 0.0, &u0, &f2);
         }
-        // column c of H1 diag(1, H2): w = diag(1, H2) e_c, then H1 w
+        // column c of H1 diag(1, H2): z = diag(1, H2) e_c, then H1 z
         const int c = l & 3;
-        double w[4];
-        w[0] = (c == 0) ? 1.0 : 0.0;
-#pragma unroll
-        for (int i = 1; i < 4; ++i)
-            w[i] = (c == 0) ? 0.0 : (((i == c) ? 1.0 : 0.0) - t2 * v2[i - 1] * v2[c - 1]);
-        double d = 0.0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) d = fma(v1[i], w[i], d);
-        d *= t1;
+        const double uc = f2 * (c == 1 ? u0 : (c == 2 ? u1 : (c == 3 ? u2 : 0.0)));
+        const double z0 = c == 0 ? 1.0 : 0.0, z1 = fma(-uc, u0, c == 1 ? 1.0 : 0.0);
+        const double z2 = fma(-uc, u1, c == 2 ? 1.0 : 0.0), z3 = fma(-uc, u2, c == 3 ? 1.0 : 0.0);
+        const double d = fma(w0, z0, fma(a1, z1, a2 * z2)) * f1;
         double* out = sc + (zhalf ? SC_Z : SC_Q) + c * 4;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) out[i] = fma(-d, v1[i], w[i]);
+        out[0] = fma(-d, w0, z0);
+        out[1] = fma(-d, a1, z1);
+        out[2] = fma(-d, a2, z2);
+        out[3] = z3;
     }
     __syncwarp(om);
     const double* Qs = sc + SC_Q;
@@ -331,7 +449,7 @@ __device__ __forceinline__ bool gen_swap_octet(int p, int q, const double* __res
         }
         // weak test on the block that must vanish: rows [q, k) x columns [0, q)
         if (ec < q && r >= q && r < k) {
-            low |= mag(na) > mag(tha) || mag(nb) > mag(thb);
+            low |= mag(na) > tha || mag(nb) > thb;
             na = 0.0;
             nb = 0.0;
         }
@@ -359,36 +477,39 @@ __device__ __forceinline__ bool gen_swap_octet(int p, int q, const double* __res
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             const int r = er + t;
-            double ea = 0.0, eb = 0.0;
+            double va = 0.0, vb = 0.0;
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                ea = fma(sc[SC_WA + a * 4 + r], Zs[a * 4 + ec], ea);
-                eb = fma(sc[SC_WB + a * 4 + r], Zs[a * 4 + ec], eb);
+                va = fma(sc[SC_WA + a * 4 + r], Zs[a * 4 + ec], va);
+                vb = fma(sc[SC_WB + a * 4 + r], Zs[a * 4 + ec], vb);
             }
-            bad |= mag(ea - DA[ec * 4 + r]) > mag(tha) || mag(eb - DB[ec * 4 + r]) > mag(thb);
+            bad |= mag(va - DA[ec * 4 + r]) > tha || mag(vb - DB[ec * 4 + r]) > thb;
         }
         if (__any_sync(om, bad)) return false;
     }
     // --- T stays upper triangular: rotate the two columns of each new 2x2
     // block (lanes 0-3: rows of NA, lanes 4-7: rows of NB, then all of Zs).
-    // The two blocks own disjoint columns, so both rotations are computed
-    // first (independent chains) and applied one after the other.
+    // The two blocks own disjoint columns: lanes 0-3 compute the rotation of
+    // the upper one, lanes 4-7 of the lower one.
     double rc[2], rs[2];
     bool act[2];
-#pragma unroll
-    for (int blk = 0; blk < 2; ++blk) {
-        const int sz = blk ? p : q, c0 = blk ? q : 0;
-        act[blk] = false;
-        rc[blk] = 1.0;
-        rs[blk] = 0.0;
+    {
+        const int sz = zhalf ? p : q, c0 = zhalf ? q : 0;
+        double cs = 1.0, sn = 0.0;
+        int rot = 0;
         if (sz == 2) {
             const double b10 = sc[SC_NB + c0 * 4 + c0 + 1], b11 = sc[SC_NB + (c0 + 1) * 4 + c0 + 1];
-            if (b10 != 0.0) {
-                const double rh = 1.0 / hypot(b10, b11);
-                act[blk] = true;
-                rc[blk] = b11 * rh;
-                rs[blk] = -b10 * rh;
+            if (!is_zero(b10)) {
+                givens64(b11, b10, &cs, &sn);
+                sn = -sn;
+                rot = 1;
             }
+        }
+#pragma unroll
+        for (int blk = 0; blk < 2; ++blk) {
+            rc[blk] = __shfl_sync(om, cs, ob + 4 * blk);
+            rs[blk] = __shfl_sync(om, sn, ob + 4 * blk);
+            act[blk] = __shfl_sync(om, rot, ob + 4 * blk) != 0;
         }
     }
     __syncwarp(om);

@@ -26,7 +26,7 @@
 
 #include "common.cuh"
 #include "ozaki.cuh"
-#include "swap_math.cuh"
+#include "seeded.cuh"
 
 #include <cuda_bf16.h>
 #include <float.h>
@@ -159,48 +159,6 @@ __device__ __forceinline__ bool sylv22_regs(const double* D, double* X) {
 // and a lane of a product warp works on two items at once); the rounding errors of whole reorderings (orthogonality, residual, swaps sent to
 // the double-double retry) are a little smaller than they were.
 // ---------------------------------------------------------------------------
-// Seeds with about 20 correct bits (PTX rcp/rsqrt.approx.ftz.f64).
-__device__ __forceinline__ double rcp_seed(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    return y;
-}
-__device__ __forceinline__ double rsqrt_seed(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    return y;
-}
-// x times 2^-1 for a normal x above the smallest binade.
-__device__ __forceinline__ double half_of(double x) {
-    return __longlong_as_double(__double_as_longlong(x) - (1LL << 52));
-}
-// x >= 0 and x == 0 (either zero) on the integer pipe.
-__device__ __forceinline__ bool nonneg(double x) {
-    return __double_as_longlong(x) >= 0 || __double_as_longlong(x) == (long long)(1ULL << 63);
-}
-__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
-// max(10 eps m, DBL_MIN), the threshold of the stability tests, as a bit
-// pattern (m >= 0).
-__device__ __forceinline__ unsigned long long thresh_bits(unsigned long long m) {
-    const unsigned long long t = abs_bits(10.0 * DBL_EPSILON * bits_double(m));
-    return t > 0x0010000000000000ULL ? t : 0x0010000000000000ULL;
-}
-// 1/x for normal x: one third-order step, y (1 + e + e^2) with e = 1 - x y
-// (the geometric series of 1 / (1 - e)).
-__device__ __forceinline__ double rcp64(double x) {
-    const double y = rcp_seed(x), e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-// sqrt(x) for normal x: one step of Goldschmidt's iteration on (sqrt, 1/(2
-// sqrt)) and a final residual correction (Markstein 2004).
-__device__ __forceinline__ double sqrt64(double x) {
-    const double y = rsqrt_seed(x);
-    double g = x * y, h = half_of(y);
-    const double r = fma(-g, h, 0.5);
-    g = fma(g, r, g);
-    h = fma(h, r, h);
-    return fma(fma(-g, g, x), h, g);
-}
 // Reflector I - f w w^T with w = (w0, a1, 1) that maps a = (a0, a1, 1) onto
 // -sign(a0) |a| e_0: w0 = a0 + sign(a0) |a|, f = 2 / |w|^2 (taken from the
 // rounded w, so that only f's own rounding touches the orthogonality).  The
@@ -219,23 +177,6 @@ __device__ __forceinline__ void apply_refl3(double w0, double w1, double f, doub
     *x1 = fma(-s, w1, *x1);
     *x2 -= s;
 }
-// x 2^(127 - eoff) as a float by truncation, and a float as a double, both on
-// the integer pipe (0 below the normal range, infinity above it).
-__device__ __forceinline__ float to_f32(double x, int eoff) {
-    const unsigned hi = __double2hiint(x), lo = __double2loint(x);
-    const int fld = (int)((hi >> 20) & 0x7ff), e = fld - eoff;
-    const unsigned b = e <= 0 || fld == 0 ? 0u
-                     : e >= 255 ? 0x7f800000u
-                                : ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-    return __uint_as_float((hi & 0x80000000u) | b);
-}
-__device__ __forceinline__ double from_f32(float x) {
-    const unsigned b = __float_as_uint(x), e = (b >> 23) & 255u;
-    if (e == 0) return 0.0;
-    return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)),
-                            (int)(b << 29));
-}
-
 // The elimination kept for the swaps whose FP32-seeded solution does not
 // converge (out of line: it is rare, and the step loop must fit the
 // instruction caches).
@@ -316,7 +257,10 @@ __device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, i
         x[1] = fmaf(m00, y10, -m10 * y00) * rdet;
         x[2] = fmaf(m11, y01, -m01 * y11) * rdet;
         x[3] = fmaf(m00, y11, -m10 * y01) * rdet;
-        return fmaxf(fmaxf(fabsf(x[0]), fabsf(x[1])), fmaxf(fabsf(x[2]), fabsf(x[3])));
+        unsigned m = 0;  // largest |x|, NaN above all
+#pragma unroll
+        for (int t = 0; t < 4; ++t) m = max(m, __float_as_uint(x[t]) & 0x7fffffffu);
+        return __uint_as_float(m);
     };
     // lane's entry (i, k) of the 2x2 matrices X and of the residual
     const int i = l & 1, k = (l >> 1) & 1;
@@ -489,28 +433,6 @@ __device__ __forceinline__ bool swap3_quad(const double* __restrict__ Sp, int ja
     z[2] = f;
     const unsigned votes = __ballot_sync(full, ok);
     return ((votes >> base) & 15u) == 15u;
-}
-
-// Givens rotation (c, s) from (t, d): (t, d) / |(t, d)|.  Values whose squares
-// leave the normal range are scaled by a power of two first.
-__device__ __forceinline__ void givens64(double t, double d, double* c, double* s) {
-    double nn = fma(t, t, d * d);
-    const unsigned e = (unsigned)__double2hiint(nn) >> 20;
-    if (e < 100u || e > 1900u) {
-        const unsigned long long bt = abs_bits(t), bd = abs_bits(d);
-        const int em = (int)((bt > bd ? bt : bd) >> 52);
-        const double sc = __hiloint2double((em < 1 ? 2045 : (em > 2045 ? 1 : 2046 - em)) << 20, 0);
-        t *= sc;
-        d *= sc;
-        nn = fma(t, t, d * d);
-    }
-    // 1 / sqrt(nn): one third-order step, y (1 + e/2 + 3 e^2 / 8) with
-    // e = 1 - nn y^2 (the binomial series of (1 - e)^(-1/2))
-    const double y = rsqrt_seed(nn);
-    const double r = fma(-(nn * y), y, 1.0);
-    const double rh = fma(y * r, fma(0.375, r, 0.5), y);
-    *c = t * rh;
-    *s = d * rh;
 }
 
 // Swap types of a step, each handled by its own warps (FP64 issue costs the
