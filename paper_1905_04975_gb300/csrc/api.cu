@@ -753,24 +753,22 @@ int gbr_eigenvectors(int n, const double* S, int ldS, const double* Q, int ldQ,
     const int ncb = (m + GN - 1) / GN;
     std::vector<int> kmax(ncb);
     for (int cb = 0; cb < ncb; ++cb) kmax[cb] = col_top[std::min(m, (cb + 1) * GN) - 1];
-    // scratch: blocks, kmax, column bounds, scalings, Y (when back-transformed),
-    // and the right-hand sides of one wave of CTAs when they do not fit shared memory
-    const bool rsm = eigvec_rhs_smem(n) != 0;
-    const int wave = rsm ? nblk : std::min(nblk, 8 * num_sms());
+    // scratch: blocks, kmax, column bounds, scalings, bounds of the right-hand
+    // sides, Y (when back-transformed)
     const size_t b_blk = align256(sizeof(int4) * nblk), b_km = align256(sizeof(int) * ncb);
     const size_t b_cm = align256(sizeof(double) * 2 * n), b_ns = align256(sizeof(int) * m);
+    const size_t b_rb = align256(sizeof(double) * nblk);
     const size_t b_y = Q ? align256(sizeof(double) * (size_t)n * m) : 0;
-    const size_t b_r = rsm ? 0 : align256(sizeof(double) * 3 * (size_t)n * wave);
     char* e = nullptr;
-    rc = pool_get(POOL_EIGVEC, b_blk + b_km + b_cm + b_ns + b_y + b_r, (void**)&e);
+    rc = pool_get(POOL_EIGVEC, b_blk + b_km + b_cm + b_ns + b_rb + b_y, (void**)&e);
     if (rc) return rc;
     int4* d_blk = (int4*)e;
     int* d_km = (int*)(e + b_blk);
     double* d_cm = (double*)(e + b_blk + b_km);
     int* d_ns = (int*)(e + b_blk + b_km + b_cm);
-    double* d_y = Q ? (double*)(e + b_blk + b_km + b_cm + b_ns) : X;
+    double* d_rb = (double*)(e + b_blk + b_km + b_cm + b_ns);
+    double* d_y = Q ? (double*)(e + b_blk + b_km + b_cm + b_ns + b_rb) : X;
     const int ldY = Q ? n : ldX;
-    double* d_r = rsm ? nullptr : (double*)(e + b_blk + b_km + b_cm + b_ns + b_y);
     GBR_CK(cudaMemcpyAsync(d_blk, blocks.data(), sizeof(int4) * nblk, cudaMemcpyHostToDevice, st), "H2D blocks");
     GBR_CK(cudaMemcpyAsync(d_km, kmax.data(), sizeof(int) * ncb, cudaMemcpyHostToDevice, st), "H2D kmax");
     if (stats) {
@@ -800,13 +798,9 @@ int gbr_eigenvectors(int n, const double* S, int ldS, const double* Q, int ldQ,
         }
     if (stats) GBR_CK(cudaEventRecord(ev[0], st), "event");
     GBR_CK(launch_colmax(n, S, ldS, d_cm, d_cm + n, st), "column bounds kernel");
-    // back substitution, in waves when the right-hand sides live in global memory
-    for (int b0 = 0; b0 < nblk; b0 += wave) {
-        const int cnt = std::min(wave, nblk - b0);
-        const int nr = std::max(0, std::min(nreal - b0, cnt));
-        GBR_CK(launch_eigvec(n, S, ldS, d_blk + b0, cnt, nr, d_y, ldY, d_cm, d_cm + n, d_r, d_ns, st),
-               "eigenvector kernel");
-    }
+    GBR_CK(launch_eigvec(n, S, ldS, sub.data(), blocks, nreal, d_blk, d_y, ldY, d_cm, d_cm + n, d_rb, d_ns,
+                         st),
+           "eigenvector kernels");
     if (stats) GBR_CK(cudaEventRecord(ev[1], st), "event");
     if (Q) GBR_CK(launch_evgemm(n, m, Q, ldQ, d_y, ldY, X, ldX, d_km, st), "back-transform kernel");
     if (stats) GBR_CK(cudaEventRecord(ev[2], st), "event");

@@ -5,6 +5,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <vector>
+
 namespace gbr {
 
 // Largest diagonal window whose packed upper-Hessenberg S window and dense
@@ -181,15 +183,16 @@ cudaError_t launch_panel_dmma(int rows, int w, double* Y, long long rs, long lon
 cudaError_t launch_panel_ozaki(int rows, int w, double* Y, long long rs, long long ks,
                                const double* Ug, unsigned char* us, int* err, int grid,
                                cudaStream_t st);
-// Eigenvectors (eigvec.cu).  blocks: (j, nb, output column, -) per selected
-// diagonal block, the nreal 1x1 blocks first; rscratch: 3 n doubles per CTA
-// of the launch when eigvec_rhs_smem(n) == 0, else unused.
-size_t eigvec_rhs_smem(int n);
+// Eigenvectors (eigvec.cu).  blocks (and its device copy d_blocks): (j, nb,
+// output column, -) per selected diagonal block, the nreal 1x1 blocks first,
+// each kind in diagonal order; sub (host): 1 where rows i, i + 1 of S form a
+// 2x2 block; rb: one double per block.
 cudaError_t launch_colmax(int n, const double* S, int ldS, double* cmA, double* cmB,
                           cudaStream_t st);
-cudaError_t launch_eigvec(int n, const double* S, int ldS, const int4* d_blocks, int nblk,
-                          int nreal, double* Y, int ldY, double* cmA, double* cmB,
-                          double* rscratch, int* nscale, cudaStream_t st);
+cudaError_t launch_eigvec(int n, const double* S, int ldS, const uint8_t* sub,
+                          const std::vector<int4>& blocks, int nreal, const int4* d_blocks,
+                          double* Y, int ldY, const double* cmA, const double* cmB, double* rb,
+                          int* nscale, cudaStream_t st);
 cudaError_t launch_evgemm(int rows, int cols, const double* A, int ldA, const double* B, int ldB,
                           double* C, int ldC, const int* d_kmax, cudaStream_t st);
 int evgemm_col_block();

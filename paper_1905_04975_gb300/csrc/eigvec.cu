@@ -4,27 +4,43 @@
 //
 //   colmax_kernel   per column c of S: max |S[i, c]| over i < c and i < c - 1
 //                   (the bounds the overflow guard multiplies with);
-//   eigvec_kernel   one CTA per selected eigenvalue (a 1x1 block, or a 2x2
-//                   block = a conjugate pair, stored as real and imaginary
-//                   column): column-oriented back substitution over the
-//                   diagonal blocks above it;
-//   evgemm_kernel   X = Q Y with FP64 tensor-core products (DMMA); a column
-//                   block of Y is nonzero only in its leading rows, so the
-//                   inner dimension stops there;
+//   evinit_kernel   the start vector of each selected eigenvalue (a 1x1 block,
+//                   or a 2x2 block = a conjugate pair, stored as real and
+//                   imaginary column), zeros elsewhere;
+//   evdiag_kernel   back substitution inside one block of up to 32 rows, one
+//                   warp per vector;
+//   evupd_kernel    the block's contribution to the rows above, one matrix
+//                   product over all vectors;
+//   evgemm_kernel   X = Q Y; a column block of Y is nonzero only in its leading
+//                   rows, so the inner dimension stops there;
 //   evnorm_kernel   max |x_i| = 1 per real vector, max(|re| + |im|) = 1 per
 //                   complex one.
 //
-// Back substitution: r = -S[0:j, B(j)] y[B(j)]; for each block B above,
-// y[B] = (S[B,B] - lambda I)^-1 r[B] (one thread), then r[0:B0] -= S[0:B0, B]
-// y[B] (all threads).  A pivot below smin = max(eps |lambda|, DBL_MIN / eps)
-// is raised to smin.  rb bounds max|r| over the remaining rows (|z| = |re| +
-// |im|); before a block is solved and before its update, the vector is
-// scaled by 2^-512 (exact) while the next value or the new bound would exceed
-// 2^900.  The right-hand side lives in shared memory when it fits.
+// Back substitution, 32 rows at a time from the bottom for all vectors that
+// reach them: Y's rows above a block hold the right-hand side r (starting at
+// zero; the start entries enter with their own block's product), the warp of
+// a vector solves y[B] = (S[B,B] - lambda I)^-1 r[B] for each diagonal block B
+// of the rows and updates the rows above B within them, and one product
+// Y[0:lo, :] -= S[0:lo, lo:hi] Y[lo:hi, :] updates everything above.  A pivot
+// below smin = max(eps |lambda|, DBL_MIN / eps) is raised to smin.  rb bounds
+// max|r| over the remaining rows (|z| = |re| + |im|); before a diagonal block
+// is solved and before its update, the vector is scaled by 2^-512 (exact)
+// while the next value or the new bound would exceed 2^900.  The bounds only
+// grow, so a warp first solves its rows without the guards and redoes them
+// with the guards if the bound at the end, or a value, is over the limit.
+//
+// What bounds it: the FP64 pipe (products at 64 cycles a warp instruction).
+// One CTA per vector with a barrier per diagonal block took 40.4 ms for the
+// 21.3 GFLOP of the n = 4000 form (0.53 TFLOP/s: a chain of about 30 FP64
+// instructions per block between two barriers); in blocks of 32 rows nearly
+// all of the work is a matrix product, 25.0 ms in all (0.85 TFLOP/s).
 #include "common.cuh"
 #include "host.h"
 
 #include <float.h>
+
+#include <algorithm>
+#include <vector>
 
 namespace gbr {
 
@@ -176,295 +192,391 @@ __device__ __forceinline__ int solve_guarded(const BlkInv& B, cd r0, cd r1, doub
     return s;
 }
 
-// One eigenvector per CTA.  blocks[b] = (j, nb, column of Y, -); Y column-
-// major (ldY), written for every row (zero below the vector's support).
-// rscratch: per-CTA right-hand side and 2x2 flags in global memory (3 n
-// doubles per CTA), used when rsm == 0; otherwise both are in dynamic shared
-// memory.  nscale[col]: the number of 2^-512 scalings.
-//
-// Pipelined by one block: while warps 1..7 apply the update of block B_t to
-// the rows below the next block, warp 0 applies it to the next block's rows
-// and lane 0 solves the next block (its pending scaling is applied at the
-// start of the following step, before anything else reads the rows).  The
-// inverses of the shifted diagonal blocks are computed 32 blocks at a time
-// by the lanes of warp 0 (one block per lane) into a ring, so that the
-// serial step of lane 0 is a few multiplications and the guards.
-template <bool CPLX>
+constexpr int EB = 32;  // rows per block of the back substitution: a lane each
+
+// A real pivot raised to smin where it is smaller.
+__device__ __forceinline__ double perturb_real(double d, double smin) {
+    return fabs(d) >= smin ? d : copysign(smin, d == 0.0 ? 1.0 : d);
+}
+
+// Start vectors: blocks[b] = (j, nb, column of Y, -); Y column-major (ldY),
+// every row written.  rb[b] = max |S[0:j, j:j+nb] y[j:j+nb]|, the bound of the
+// first right-hand side.
 __global__ void __launch_bounds__(EV_THREADS)
-eigvec_kernel(int n, const double* __restrict__ S, int ldS, const int4* __restrict__ blocks,
-              double* __restrict__ Y, int ldY, const double* __restrict__ cmA,
-              const double* __restrict__ cmB, double* __restrict__ rscratch, int rsm,
+evinit_kernel(int n, const double* __restrict__ S, int ldS, const int4* __restrict__ blocks,
+              double* __restrict__ Y, int ldY, const double* __restrict__ cmA, double* __restrict__ rb,
               int* __restrict__ nscale) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[EV_THREADS / 32];
-    __shared__ cd xs[2][2];
-    __shared__ int pend[2];
-    __shared__ BlkInv ring[32];
-    __shared__ int ring_b0[33];  // block starts of the ring's blocks (entry 32: one past)
-    __shared__ int ring_first, ring_count;
     const int4 bk = blocks[blockIdx.x];
-    const int j = bk.x, nb = bk.y, col = bk.z, top = j + nb;
-    if ((nb == 2) != CPLX) return;  // launched per kind
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int j = bk.x, nb = bk.y, col = bk.z, tid = threadIdx.x;
     double* yr = Y + (size_t)col * ldY;
-    double* yi = CPLX ? Y + (size_t)(col + 1) * ldY : nullptr;
-    double* rr = rsm ? reinterpret_cast<double*>(smem_raw) : rscratch + (size_t)blockIdx.x * 3 * n;
-    double* ri = rr + n;  // imaginary parts (complex vectors)
-    uint8_t* sub = rsm ? smem_raw + sizeof(double) * 2 * (size_t)n
-                       : reinterpret_cast<uint8_t*>(ri + n);  // 2x2 flag of rows i, i+1
-    // eigenvalue and start vector
-    double lr, li = 0.0, y1i = 0.0;
-    if (!CPLX) {
-        lr = __ldg(&S[cm(j, j, ldS)]);
-    } else {
-        const double a = __ldg(&S[cm(j, j, ldS)]), b = __ldg(&S[cm(j, j + 1, ldS)]);
-        const double c = __ldg(&S[cm(j + 1, j, ldS)]);
-        const double w = sqrt(-b * c);
-        lr = a;
-        li = w;
-        y1i = w / b;
-    }
-    const double smin = fmax(DBL_EPSILON * (fabs(lr) + fabs(li)), DBL_MIN / DBL_EPSILON);
-    // y rows >= j; r = -S[0:j, j:top] y[j:top]; the 2x2 pattern above j
-    for (int i = j + tid; i < n; i += EV_THREADS) {
-        yr[i] = (i == j) ? 1.0 : 0.0;
-        if (CPLX) yi[i] = (i == j + 1) ? y1i : 0.0;
-    }
-    double m = 0.0;
-    for (int i = tid; i < j; i += EV_THREADS) {
-        const double s0 = __ldg(&S[cm(i, j, ldS)]);
-        sub[i] = (i + 1 < j && __ldg(&S[cm(i + 1, i, ldS)]) != 0.0) ? 1 : 0;
-        if (!CPLX) {
-            rr[i] = -s0;
-            m = fmax(m, fabs(s0));
-        } else {
-            const double s1 = __ldg(&S[cm(i, j + 1, ldS)]);
-            rr[i] = -s0;
-            ri[i] = -s1 * y1i;
-            m = fmax(m, fabs(s0) + fabs(s1 * y1i));
-        }
-    }
-    double rb = block_max(m, red);  // maintained by thread 0 only
-    if (j == 0) {
-        if (tid == 0 && nscale) {
+    if (nb == 1) {
+        for (int i = tid; i < n; i += EV_THREADS) yr[i] = i == j ? 1.0 : 0.0;
+        if (tid == 0) {
+            rb[blockIdx.x] = cmA[j];
             nscale[col] = 0;
-            if (CPLX) nscale[col + 1] = 0;
         }
         return;
     }
-    auto block_below = [&](int e) { return (e >= 2 && sub[e - 2]) ? e - 2 : e - 1; };
-    auto colbound = [&](int b0, int k) { return (k == 1) ? cmA[b0] : fmax(cmA[b0], cmB[b0 + 1]); };
-    // warp 0: the inverses of the next (up to) 32 blocks below e
-    auto refill = [&](int e, int first) {
-        if (lane == 0) {
-            int cnt = 0, t = e;
-            while (cnt < 32 && t > 0) {
-                const int b = block_below(t);
-                ring_b0[cnt++] = b;
-                t = b;
-            }
-            ring_b0[cnt] = t;
-            ring_count = cnt;
-            ring_first = first;
-        }
-        __syncwarp();
-        if (lane < ring_count) {
-            const int b = ring_b0[lane], e2 = lane ? ring_b0[lane - 1] : e;
-            ring[lane] = block_inverse(S, ldS, b, e2 - b, lr, li, smin);
-        }
-        __syncwarp();
-    };
-    int b1 = j, b0 = block_below(j);
-    if (warp == 0) {
-        refill(j, 0);
-        if (lane == 0) {
-            const BlkInv& Bi = ring[0];
-            const int k = Bi.k;
-            cd x0, x1;
-            const int s = solve_guarded<CPLX>(
-                Bi, cd{rr[b0], CPLX ? ri[b0] : 0.0},
-                cd{k == 2 ? rr[b0 + 1] : 0.0, (CPLX && k == 2) ? ri[b0 + 1] : 0.0},
-                b0 > 0 ? colbound(b0, k) : 0.0, rb, x0, x1);
-            xs[0][0] = x0;
-            xs[0][1] = x1;
-            pend[0] = s;
-            yr[b0] = x0.re;
-            if (CPLX) yi[b0] = x0.im;
-            if (k == 2) {
-                yr[b0 + 1] = x1.re;
-                if (CPLX) yi[b0 + 1] = x1.im;
-            }
+    const double b = __ldg(&S[cm(j, j + 1, ldS)]), c = __ldg(&S[cm(j + 1, j, ldS)]);
+    const double y1i = sqrt(-b * c) / b;
+    double m = 0.0;
+    for (int i = tid; i < n; i += EV_THREADS) {
+        yr[i] = i == j ? 1.0 : 0.0;
+        yr[ldY + (size_t)i] = i == j + 1 ? y1i : 0.0;
+        if (i < j) m = fmax(m, fabs(__ldg(&S[cm(i, j, ldS)])) + fabs(__ldg(&S[cm(i, j + 1, ldS)]) * y1i));
+    }
+    m = block_max(m, red);
+    if (tid == 0) {
+        rb[blockIdx.x] = m;
+        nscale[col] = nscale[col + 1] = 0;
+    }
+}
+
+// The rows [lo, hi) (at most EB, cutting no 2x2 block) of one vector, by one
+// warp; lane = row.  D: the diagonal block S[lo:hi, lo:hi] in shared memory
+// (column-major, ld EB + 1); cb: per row that starts a diagonal block, its
+// column bound (0 for the top of S).
+template <bool CPLX>
+__device__ __forceinline__ void diag_vector(const double* __restrict__ S, int ldS, int lo, int hi,
+                                            const double* D, const double* cb, int4 bk, double* Y,
+                                            int ldY, double* rbp, int* __restrict__ nscale) {
+    constexpr int LD = EB + 1;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, rows = hi - lo;
+    const int j = bk.x, top = min(j, hi) - lo;  // rows [0, top) of the block are solved
+    if (top <= 0) return;
+    double* yr = Y + (size_t)bk.z * ldY + lo;
+    double* yi = yr + ldY;
+    double lr = __ldg(&S[cm(j, j, ldS)]), li = 0.0, y1i = 0.0;
+    if (CPLX) {
+        const double b = __ldg(&S[cm(j, j + 1, ldS)]), c = __ldg(&S[cm(j + 1, j, ldS)]);
+        li = sqrt(-b * c);
+        y1i = li / b;
+    }
+    const double smin = fmax(DBL_EPSILON * (fabs(lr) + fabs(li)), DBL_MIN / DBL_EPSILON);
+    const bool act = lane < top;
+    // 2x2 blocks: bit i of two = rows i, i + 1 form one
+    const unsigned two = __ballot_sync(full, lane + 1 < rows && D[lane * LD + lane + 1] != 0.0);
+    const bool second = lane > 0 && ((two >> (lane - 1)) & 1u);
+    const int k = (two >> lane) & 1u ? 2 : 1;
+    // the right-hand side of this row
+    double re0 = 0.0, im0 = 0.0;
+    if (act) {
+        if (j < hi) {
+            re0 = -D[(j - lo) * LD + lane];
+            if (CPLX) im0 = -D[(j - lo + 1) * LD + lane] * y1i;
+        } else {
+            re0 = yr[lane];
+            if (CPLX) im0 = yi[lane];
         }
     }
-    __syncthreads();
-    int cur = 0, step = 0, nsc = 0;
-    if (tid == 0) nsc = pend[0];
-    while (b0 > 0) {
-        const int k = b1 - b0;
-        const int s = pend[cur];
-        const cd x0 = xs[cur][0], x1 = xs[cur][1];
-        const int c1 = b0, c0 = block_below(b0), kn = c1 - c0;  // next block [c0, c1)
-        double f = 1.0;
-        if (s) {  // rare: the rows already computed move to the new scale
-            for (int t = 0; t < s; ++t) f *= EV_SHRINK;
-            for (int i = b1 + tid; i < top; i += EV_THREADS) {
-                yr[i] *= f;
-                if (CPLX) yi[i] *= f;
+    // x of this row = c0 r[b] + c1 r[b + 1] for its block's rows b, b + 1
+    cd c0{0.0, 0.0}, c1{0.0, 0.0};
+    BlkInv B;
+    if (act && !second) {
+        if (CPLX) {
+            B = block_inverse(S, ldS, lo + lane, k, lr, li, smin);
+        } else {
+            const double m00 = D[lane * LD + lane] - lr;
+            B.b0 = lo + lane;
+            B.k = k;
+            B.inv[0] = B.inv[1] = B.inv[2] = B.inv[3] = cd{0.0, 0.0};
+            if (k == 1) {
+                B.inv[0].re = 1.0 / perturb_real(m00, smin);
+            } else {
+                const double m01 = D[(lane + 1) * LD + lane], m10 = D[lane * LD + lane + 1];
+                const double m11 = D[(lane + 1) * LD + lane + 1] - lr;
+                const double mx = fmax(fmax(fabs(m00), fabs(m01)), fmax(fabs(m10), fabs(m11)));
+                const double rd = 1.0 / perturb_real(fma(m00, m11, -m01 * m10), smin * fmax(mx, smin));
+                B.inv[0].re = m11 * rd;
+                B.inv[1].re = -m01 * rd;
+                B.inv[2].re = -m10 * rd;
+                B.inv[3].re = m00 * rd;
             }
         }
-        if (warp == 0) {
-            // the next block's rows: scale, update by B, then solve (lane 0)
-            if (lane < kn) {
-                const int i = c0 + lane;
-                const double s0 = __ldg(&S[cm(i, b0, ldS)]);
-                const double s1 = (k == 2) ? __ldg(&S[cm(i, b0 + 1, ldS)]) : 0.0;
-                double v = s ? rr[i] * f : rr[i];
-                v = fma(-s0, x0.re, v);
-                if (k == 2) v = fma(-s1, x1.re, v);
-                rr[i] = v;
-                if (CPLX) {
-                    double u = s ? ri[i] * f : ri[i];
-                    u = fma(-s0, x0.im, u);
-                    if (k == 2) u = fma(-s1, x1.im, u);
-                    ri[i] = u;
-                }
-            }
-            const int q = step + 1;  // index of the next block, counted from the eigenvalue
-            if (q - ring_first >= ring_count) refill(c1, q);
-            else __syncwarp();
-            if (lane == 0) {
-                const BlkInv& Bi = ring[q - ring_first];
-                cd y0, y1;
-                const int sn = solve_guarded<CPLX>(
-                    Bi, cd{rr[c0], CPLX ? ri[c0] : 0.0},
-                    cd{kn == 2 ? rr[c0 + 1] : 0.0, (CPLX && kn == 2) ? ri[c0 + 1] : 0.0},
-                    c0 > 0 ? colbound(c0, kn) : 0.0, rb, y0, y1);
-                xs[cur ^ 1][0] = y0;
-                xs[cur ^ 1][1] = y1;
-                pend[cur ^ 1] = sn;
-                nsc += sn;
-                yr[c0] = y0.re;
-                if (CPLX) yi[c0] = y0.im;
-                if (kn == 2) {
-                    yr[c0 + 1] = y1.re;
-                    if (CPLX) yi[c0 + 1] = y1.im;
-                }
-            }
-        } else if (s) {
-            // rows below the next block: scale, update by B
-            for (int i = tid - 32; i < c0; i += EV_THREADS - 32) {
-                const double s0 = __ldg(&S[cm(i, b0, ldS)]);
-                const double s1 = (k == 2) ? __ldg(&S[cm(i, b0 + 1, ldS)]) : 0.0;
-                double v = fma(-s0, x0.re, rr[i] * f);
-                if (k == 2) v = fma(-s1, x1.re, v);
-                rr[i] = v;
-                if (CPLX) {
-                    double u = fma(-s0, x0.im, ri[i] * f);
-                    if (k == 2) u = fma(-s1, x1.im, u);
-                    ri[i] = u;
-                }
-            }
-        } else if (k == 1) {
-            for (int i = tid - 32; i < c0; i += EV_THREADS - 32) {
-                const double sv = __ldg(&S[cm(i, b0, ldS)]);
-                rr[i] = fma(-sv, x0.re, rr[i]);
-                if (CPLX) ri[i] = fma(-sv, x0.im, ri[i]);
+        c0 = B.inv[0];
+        c1 = B.inv[1];
+    }
+    {
+        const double a = __shfl_up_sync(full, B.inv[2].re, 1), b = __shfl_up_sync(full, B.inv[3].re, 1);
+        if (second) c0.re = a, c1.re = b;
+        if (CPLX) {
+            const double c = __shfl_up_sync(full, B.inv[2].im, 1), d = __shfl_up_sync(full, B.inv[3].im, 1);
+            if (second) c0.im = c, c1.im = d;
+        }
+    }
+    double re = re0, im = im0, xr = 0.0, xi = 0.0;
+    for (int e = top; e > 0;) {
+        const int kb = e >= 2 && ((two >> (e - 2)) & 1u) ? 2 : 1, b = e - kb;
+        double x, z = 0.0;
+        if (kb == 1) {
+            if (CPLX) {
+                const cd v = cmul(c0, cd{re, im});
+                x = v.re;
+                z = v.im;
+            } else {
+                x = c0.re * re;
             }
         } else {
-            for (int i = tid - 32; i < c0; i += EV_THREADS - 32) {
-                const double s0 = __ldg(&S[cm(i, b0, ldS)]), s1 = __ldg(&S[cm(i, b0 + 1, ldS)]);
-                rr[i] = fma(-s1, x1.re, fma(-s0, x0.re, rr[i]));
-                if (CPLX) ri[i] = fma(-s1, x1.im, fma(-s0, x0.im, ri[i]));
+            const double r0 = __shfl_sync(full, re, b), r1 = __shfl_sync(full, re, b + 1);
+            if (CPLX) {
+                const double i0 = __shfl_sync(full, im, b), i1 = __shfl_sync(full, im, b + 1);
+                const cd v = cmul(c0, cd{r0, i0}), w = cmul(c1, cd{r1, i1});
+                x = v.re + w.re;
+                z = v.im + w.im;
+            } else {
+                x = fma(c1.re, r1, c0.re * r0);
             }
         }
-        __syncthreads();
-        b1 = c1;
-        b0 = c0;
-        cur ^= 1;
-        ++step;
-    }
-    // the last block's pending scaling: the rows already computed below it
-    {
-        const int s = pend[cur];
-        if (s) {
-            double f = 1.0;
-            for (int t = 0; t < s; ++t) f *= EV_SHRINK;
-            for (int i = b1 + tid; i < top; i += EV_THREADS) {
-                yr[i] *= f;
-                if (CPLX) yi[i] *= f;
+        if (lane >= b && lane < e) {
+            xr = x;
+            xi = z;
+        }
+        const double x0 = __shfl_sync(full, x, b), z0 = CPLX ? __shfl_sync(full, z, b) : 0.0;
+        if (kb == 2) {
+            const double x1 = __shfl_sync(full, x, b + 1), s1 = D[(b + 1) * LD + lane];
+            if (lane < b) re = fma(-s1, x1, re);
+            if (CPLX) {
+                const double z1 = __shfl_sync(full, z, b + 1);
+                if (lane < b) im = fma(-s1, z1, im);
             }
         }
+        const double s0 = D[b * LD + lane];
+        if (lane < b) {
+            re = fma(-s0, x0, re);
+            if (CPLX) im = fma(-s0, z0, im);
+        }
+        e = b;
     }
-    if (tid == 0 && nscale) {
-        nscale[col] = nsc;
-        if (CPLX) nscale[col + 1] = nsc;
+    // would a guard have acted?  (the bound grows with every block)
+    double rb = *rbp;
+    const double mag = CPLX ? fabs(xr) + fabs(xi) : fabs(xr);
+    const double mag1 = __shfl_down_sync(full, mag, 1);
+    double inc = act && !second ? (double)k * cb[lane] * (k == 2 ? fmax(mag, mag1) : mag) : 0.0;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) inc += __shfl_xor_sync(full, inc, o);
+    const bool fine = (!act || mag <= EV_BIG) && rb + inc <= EV_BIG;  // (NaN is not)
+    if (__all_sync(full, fine)) {
+        if (act) {
+            yr[lane] = xr;
+            if (CPLX) yi[lane] = xi;
+        }
+        if (lane == 0) *rbp = rb + inc;
+        return;
+    }
+    // guarded: block by block, lane 0 decides the scalings
+    re = re0;
+    im = im0;
+    xr = xi = 0.0;
+    int s = 0;
+    for (int e = top; e > 0;) {
+        const int kb = e >= 2 && ((two >> (e - 2)) & 1u) ? 2 : 1, b = e - kb, b2 = b + kb - 1;
+        const cd r0{__shfl_sync(full, re, b), __shfl_sync(full, im, b)};
+        cd r1{__shfl_sync(full, re, b2), __shfl_sync(full, im, b2)};
+        if (kb == 1) r1 = cd{0.0, 0.0};
+        BlkInv Bb;
+        Bb.b0 = lo + b;
+        Bb.k = kb;
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            Bb.inv[t] = cd{__shfl_sync(full, B.inv[t].re, b), __shfl_sync(full, B.inv[t].im, b)};
+        cd x0{0.0, 0.0}, x1{0.0, 0.0};
+        int sb = 0;
+        if (lane == 0) sb = solve_guarded<CPLX>(Bb, r0, r1, cb[b], rb, x0, x1);
+        sb = __shfl_sync(full, sb, 0);
+        x0 = cd{__shfl_sync(full, x0.re, 0), __shfl_sync(full, x0.im, 0)};
+        x1 = cd{__shfl_sync(full, x1.re, 0), __shfl_sync(full, x1.im, 0)};
+        for (int t = 0; t < sb; ++t) {
+            re *= EV_SHRINK;
+            im *= EV_SHRINK;
+            xr *= EV_SHRINK;
+            xi *= EV_SHRINK;
+        }
+        s += sb;
+        if (lane == b) xr = x0.re, xi = x0.im;
+        if (kb == 2 && lane == b + 1) xr = x1.re, xi = x1.im;
+        if (lane < b) {
+            const double s0 = D[b * LD + lane], s1 = kb == 2 ? D[(b + 1) * LD + lane] : 0.0;
+            re = fma(-s1, x1.re, fma(-s0, x0.re, re));
+            if (CPLX) im = fma(-s1, x1.im, fma(-s0, x0.im, im));
+        }
+        e = b;
+    }
+    if (act) {
+        yr[lane] = xr;
+        if (CPLX) yi[lane] = xi;
+    }
+    if (lane == 0) *rbp = rb;
+    if (s == 0) return;
+    // the vector's other rows move to the new scale: the right-hand side
+    // above, the solution below (its support ends with its own block)
+    double f = 1.0;
+    for (int t = 0; t < s; ++t) f *= EV_SHRINK;
+    const int end = j + bk.y - lo;
+    for (int i = lane - lo; i < end; i += 32) {
+        if (i >= 0 && i < top) continue;
+        yr[i] *= f;
+        if (CPLX) yi[i] *= f;
+    }
+    if (lane == 0) {
+        nscale[bk.z] += s;
+        if (CPLX) nscale[bk.z + 1] += s;
+    }
+}
+
+constexpr int DIAG_WARPS = 4;
+
+// The vectors blocks[r0, r0 + nr) (real) and blocks[c0, c0 + nc) (complex),
+// those whose block lies at or below row lo, one per warp.
+__global__ void __launch_bounds__(32 * DIAG_WARPS)
+evdiag_kernel(const double* __restrict__ S, int ldS, int lo, int hi, const int4* __restrict__ blocks,
+              int r0, int nr, int c0, int nc, double* __restrict__ Y, int ldY,
+              const double* __restrict__ cmA, const double* __restrict__ cmB, double* __restrict__ rb,
+              int* __restrict__ nscale) {
+    __shared__ double D[EB * (EB + 1)], cb[EB];
+    const int rows = hi - lo, tid = threadIdx.x;
+    for (int i = tid; i < EB * EB; i += 32 * DIAG_WARPS) {
+        const int r = i & (EB - 1), c = i / EB;
+        D[c * (EB + 1) + r] = r < rows && c < rows && r <= c + 1 ? __ldg(&S[cm(lo + r, lo + c, ldS)]) : 0.0;
+    }
+    __syncthreads();
+    if (tid < EB) {
+        const bool two = tid + 1 < rows && D[tid * (EB + 1) + tid + 1] != 0.0;
+        cb[tid] = tid >= rows || lo + tid == 0 ? 0.0
+                  : two ? fmax(cmA[lo + tid], cmB[lo + tid + 1]) : cmA[lo + tid];
+    }
+    __syncthreads();
+    const int v = blockIdx.x * DIAG_WARPS + (tid >> 5);
+    if (v < nr)
+        diag_vector<false>(S, ldS, lo, hi, D, cb, blocks[r0 + v], Y, ldY, rb + r0 + v, nscale);
+    else if (v < nr + nc)
+        diag_vector<true>(S, ldS, lo, hi, D, cb, blocks[c0 + v - nr], Y, ldY, rb + c0 + v - nr, nscale);
+}
+
+// C (rows x cols) -= A (rows x K) B (K x cols), column-major, K <= EB; C and B
+// are rows of the same columns of Y.  Tiles of 32 x 64, 4 x 4 per thread: the
+// FP64 pipe needs 64 cycles for a warp's FMA, so operand traffic is no
+// concern and small tiles keep the last wave short (a tile alone on an SM
+// takes 16 us).
+constexpr int UM = 32, UN = 64, LDU = UN + 2;
+
+__global__ void __launch_bounds__(128)
+evupd_kernel(int rows, int cols, int K, const double* __restrict__ A, int ldA, const double* B, int ldB,
+             double* C, int ldC) {
+    __shared__ __align__(16) double As[EB * UM], Bs[EB * LDU];
+    const int r0 = blockIdx.x * UM, c0 = blockIdx.y * UN;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rg = (lane & 7) * 4, cg = (warp * 4 + (lane >> 3)) * 2;  // columns cg, cg + 1, cg + 32, cg + 33
+    double acc[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int c = c0 + cg + (u & 1) + 32 * (u >> 1);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            acc[r][u] = r0 + rg + r < rows && c < cols ? C[cm(r0 + rg + r, c, ldC)] : 0.0;
+    }
+    for (int i = tid; i < EB * UM; i += 128) {
+        const int r = i & (UM - 1), k = i / UM;
+        As[k * UM + r] = r0 + r < rows && k < K ? __ldg(&A[cm(r0 + r, k, ldA)]) : 0.0;
+    }
+    for (int i = tid; i < EB * UN; i += 128) {
+        const int k = i & (EB - 1), c = i / EB;
+        Bs[k * LDU + c] = k < K && c0 + c < cols ? B[cm(k, c0 + c, ldB)] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < EB; ++k) {
+        double a[4], b[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const double2 x = *reinterpret_cast<const double2*>(&As[k * UM + rg + 2 * h]);
+            const double2 y = *reinterpret_cast<const double2*>(&Bs[k * LDU + cg + 32 * h]);
+            a[2 * h] = x.x;
+            a[2 * h + 1] = x.y;
+            b[2 * h] = y.x;
+            b[2 * h + 1] = y.y;
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[r][u] = fma(-a[r], b[u], acc[r][u]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int c = c0 + cg + (u & 1) + 32 * (u >> 1);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (r0 + rg + r < rows && c < cols) C[cm(r0 + rg + r, c, ldC)] = acc[r][u];
     }
 }
 
 // C (rows x cols) = A (rows x K) B (K x cols), column-major, K of column
-// block cb limited to kmax[cb] (the vectors' support); DMMA m8n8k4.
+// block cb limited to kmax[cb] (the vectors' support).  FP64 FMAs in register
+// tiles (4 x 8 per thread): both this and the tensor-core form (DMMA) are
+// bound by the same FP64 pipe, and the FMAs reach the higher rate (the n = 4000
+// form's 66 GFLOP: 56.2 ms, 1.18 TFLOP/s; with DMMA 67.9 ms, 0.97).  The column blocks with the longest
+// sums are started first, so that the last wave is short.
 constexpr int GM = 64, GN = 128, GK = 32;
-constexpr int LDA_S = GK + 4, LDB_S = GN + 8;
-constexpr size_t kGemmSmem = sizeof(double) * ((size_t)GM * LDA_S + (size_t)GK * LDB_S);
-
-__device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};\n"
-                 : "+d"(c0), "+d"(c1)
-                 : "d"(a), "d"(b));
-}
+constexpr int LDA_S = GM + 2, LDB_S = GN + 2;
+constexpr size_t kGemmSmem = sizeof(double) * (size_t)GK * (LDA_S + LDB_S);
 
 __global__ void __launch_bounds__(256)
 evgemm_kernel(int rows, int cols, const double* __restrict__ A, int ldA,
               const double* __restrict__ B, int ldB, double* __restrict__ C, int ldC,
               const int* __restrict__ kmax) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double* As = reinterpret_cast<double*>(smem_raw);  // GM x LDA_S, row-major (k contiguous)
-    double* Bs = As + GM * LDA_S;                       // GK x LDB_S, row-major (n contiguous)
-    const int r0 = blockIdx.x * GM, c0 = blockIdx.y * GN;
-    const int K = kmax[blockIdx.y];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
-    double acc[8][2][2];
+    double* As = reinterpret_cast<double*>(smem_raw);  // GK x LDA_S (rows contiguous)
+    double* Bs = As + GK * LDA_S;                       // GK x LDB_S (columns contiguous)
+    const int cb = gridDim.y - 1 - blockIdx.y;
+    const int r0 = blockIdx.x * GM, c0 = cb * GN;
+    const int K = kmax[cb];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rg = ((warp & 1) * 8 + (lane & 7)) * 4;   // rows rg .. rg + 3
+    const int cg = ((warp >> 1) * 4 + (lane >> 3)) * 2;  // columns cg + {0, 1} + 32 h, h = 0 .. 3
+    double acc[4][8];
 #pragma unroll
-    for (int rt = 0; rt < 8; ++rt)
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int ct = 0; ct < 2; ++ct) acc[rt][ct][0] = acc[rt][ct][1] = 0.0;
+        for (int u = 0; u < 8; ++u) acc[r][u] = 0.0;
     for (int k0 = 0; k0 < K; k0 += GK) {
         __syncthreads();
         for (int i = tid; i < GM * GK; i += 256) {
             const int r = i % GM, k = i / GM;
-            As[r * LDA_S + k] = (r0 + r < rows && k0 + k < K) ? __ldg(&A[cm(r0 + r, k0 + k, ldA)]) : 0.0;
+            As[k * LDA_S + r] = (r0 + r < rows && k0 + k < K) ? __ldg(&A[cm(r0 + r, k0 + k, ldA)]) : 0.0;
         }
         for (int i = tid; i < GK * GN; i += 256) {
             const int k = i % GK, c = i / GK;
             Bs[k * LDB_S + c] = (c0 + c < cols && k0 + k < K) ? __ldg(&B[cm(k0 + k, c0 + c, ldB)]) : 0.0;
         }
         __syncthreads();
-        const int cw = warp * 16;
+#pragma unroll 4
+        for (int k = 0; k < GK; ++k) {
+            double a[4], b[8];
 #pragma unroll
-        for (int kk = 0; kk < GK; kk += 4) {
-            double a[8], bb[2];
+            for (int h = 0; h < 2; ++h) {
+                const double2 x = *reinterpret_cast<const double2*>(&As[k * LDA_S + rg + 2 * h]);
+                a[2 * h] = x.x;
+                a[2 * h + 1] = x.y;
+            }
 #pragma unroll
-            for (int rt = 0; rt < 8; ++rt) a[rt] = As[(rt * 8 + gid) * LDA_S + kk + tig];
+            for (int h = 0; h < 4; ++h) {
+                const double2 y = *reinterpret_cast<const double2*>(&Bs[k * LDB_S + cg + 32 * h]);
+                b[2 * h] = y.x;
+                b[2 * h + 1] = y.y;
+            }
 #pragma unroll
-            for (int ct = 0; ct < 2; ++ct) bb[ct] = Bs[(kk + tig) * LDB_S + cw + ct * 8 + gid];
+            for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int rt = 0; rt < 8; ++rt)
-#pragma unroll
-                for (int ct = 0; ct < 2; ++ct) dmma(acc[rt][ct][0], acc[rt][ct][1], a[rt], bb[ct]);
+                for (int u = 0; u < 8; ++u) acc[r][u] = fma(a[r], b[u], acc[r][u]);
         }
     }
-    // acc[rt][ct][v]: row rt*8 + gid, column warp*16 + ct*8 + 2*tig + v
 #pragma unroll
-    for (int rt = 0; rt < 8; ++rt) {
-        const int r = r0 + rt * 8 + gid;
-        if (r >= rows) continue;
+    for (int u = 0; u < 8; ++u) {
+        const int c = c0 + cg + (u & 1) + 32 * (u >> 1);
 #pragma unroll
-        for (int ct = 0; ct < 2; ++ct)
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-                const int c = c0 + warp * 16 + ct * 8 + 2 * tig + v;
-                if (c < cols) C[cm(r, c, ldC)] = acc[rt][ct][v];
-            }
+        for (int r = 0; r < 4; ++r)
+            if (r0 + rg + r < rows && c < cols) C[cm(r0 + rg + r, c, ldC)] = acc[r][u];
     }
 }
 
@@ -494,13 +606,6 @@ cudaError_t smem_attr(K kernel, size_t bytes) {
 
 }  // namespace
 
-// Shared memory per CTA for the right-hand side of an n x n problem
-// (complex: 2 n doubles); 0 if it does not fit and global scratch is used.
-size_t eigvec_rhs_smem(int n) {
-    const size_t b = sizeof(double) * 2 * (size_t)n + (size_t)n + 16;
-    return b <= 96 * 1024 ? b : 0;
-}
-
 cudaError_t launch_colmax(int n, const double* S, int ldS, double* cmA, double* cmB,
                           cudaStream_t st) {
     if (n == 0) return cudaSuccess;
@@ -508,25 +613,48 @@ cudaError_t launch_colmax(int n, const double* S, int ldS, double* cmA, double* 
     return cudaGetLastError();
 }
 
-cudaError_t launch_eigvec(int n, const double* S, int ldS, const int4* d_blocks, int nblk,
-                          int nreal, double* Y, int ldY, double* cmA, double* cmB,
-                          double* rscratch, int* nscale, cudaStream_t st) {
+cudaError_t launch_eigvec(int n, const double* S, int ldS, const uint8_t* sub,
+                          const std::vector<int4>& blocks, int nreal, const int4* d_blocks,
+                          double* Y, int ldY, const double* cmA, const double* cmB, double* rb,
+                          int* nscale, cudaStream_t st) {
+    const int nblk = (int)blocks.size();
     if (n == 0 || nblk == 0) return cudaSuccess;
-    cudaError_t e;
-    const size_t sm = eigvec_rhs_smem(n);
-    e = smem_attr(eigvec_kernel<false>, sm);
+    evinit_kernel<<<nblk, EV_THREADS, 0, st>>>(n, S, ldS, d_blocks, Y, ldY, cmA, rb, nscale);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = smem_attr(eigvec_kernel<true>, sm);
-    if (e != cudaSuccess) return e;
-    // blocks are ordered real ones first (nreal of them), then the pairs
-    if (nreal > 0)
-        eigvec_kernel<false><<<nreal, EV_THREADS, sm, st>>>(n, S, ldS, d_blocks, Y, ldY, cmA, cmB,
-                                                           rscratch, sm ? 1 : 0, nscale);
-    if (nblk > nreal)
-        eigvec_kernel<true><<<nblk - nreal, EV_THREADS, sm, st>>>(
-            n, S, ldS, d_blocks + nreal, Y, ldY, cmA, cmB,
-            rscratch ? rscratch + (size_t)nreal * 3 * n : nullptr, sm ? 1 : 0, nscale);
-    return cudaGetLastError();
+    // the columns of Y end with the last block of either kind
+    int m = 0;
+    for (int i : {nreal - 1, nblk - 1})
+        if (i >= 0) m = std::max(m, blocks[i].z + blocks[i].y);
+    for (int hi = n; hi > 0;) {
+        int lo = std::max(0, hi - EB);
+        if (lo > 0 && sub[lo - 1]) ++lo;  // a 2x2 block starts at lo - 1
+        // vectors whose block lies at or below lo, their first column
+        const auto at = [&](int f, int l) {
+            return (int)(std::lower_bound(blocks.begin() + f, blocks.begin() + l, lo,
+                                          [](const int4& b, int x) { return b.x < x; }) -
+                         blocks.begin());
+        };
+        const int r0 = at(0, nreal), c0 = at(nreal, nblk);
+        const int nr = nreal - r0, nc = nblk - c0;
+        int col = m;
+        if (nr > 0) col = std::min(col, blocks[r0].z);
+        if (nc > 0) col = std::min(col, blocks[c0].z);
+        if (nr + nc > 0) {
+            evdiag_kernel<<<(nr + nc + DIAG_WARPS - 1) / DIAG_WARPS, 32 * DIAG_WARPS, 0, st>>>(
+                S, ldS, lo, hi, d_blocks, r0, nr, c0, nc, Y, ldY, cmA, cmB, rb, nscale);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if (lo > 0) {
+                const dim3 grid((lo + UM - 1) / UM, (m - col + UN - 1) / UN);
+                double* Yc = Y + (size_t)col * ldY;
+                evupd_kernel<<<grid, 128, 0, st>>>(lo, m - col, hi - lo, S + (size_t)lo * ldS, ldS, Yc + lo,
+                                                   ldY, Yc, ldY);
+                if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            }
+        }
+        hi = lo;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_evgemm(int rows, int cols, const double* A, int ldA, const double* B, int ldB,
