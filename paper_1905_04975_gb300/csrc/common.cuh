@@ -20,7 +20,7 @@ constexpr int WMAX_WIDE = 256;
 constexpr size_t WIDE_SP_STRIDE = ((size_t)(WMAX_WIDE * (WMAX_WIDE + 3)) / 2 + 31) & ~(size_t)31;
 
 // Split-precision (Ozaki) updates: OZ_SLICES signed 8-bit digit slices per
-// FP64 operand; one window's U slices take OZ_USLICE_BYTES (bf16 digits
+// FP64 operand; one window's U slices take OZ_USLICE_BYTES (fp16 digits
 // [slice][column n][row k], then one int exponent per column).
 constexpr int OZ_SLICES = 7;
 constexpr size_t OZ_UDIG_ELEMS = (size_t)OZ_SLICES * WMAX * WMAX;

@@ -11,8 +11,10 @@
 //
 //     V = d1 2^48 + d2 2^40 + ... + d7,   d2..d7 in [-128, 127], d1 in [-128, 128],
 //
-// computed from G = V + 0x808080808080: d1 = G >> 48 (arithmetic), dp =
-// byte (7 - p) of G minus 128.  Digits are exact in bf16.
+// computed from G = V + 0x80808080808080: d1 = (G >> 48) - 128, dp = byte
+// (7 - p) of G minus 128.  Digits are exact in fp16 (and in bf16; fp16 is used
+// because 1024 + a byte is one of its numbers, so that two digits are made by
+// a byte permute, a bit operation and one packed addition).
 //
 // Products.  For a K <= 128 contraction every slice product A_p B_q has
 // integer entries of magnitude <= 128^2 * 128 = 2^21; the products on one
@@ -22,8 +24,7 @@
 // order of d, so that the products of one Y slice p with the U slices
 // q = 1..8-p hit consecutive accumulators and run as one or two MMAs of N up
 // to 256 (the U slices are stacked along N).  The epilogue converts the
-// accumulators to integers, combines them by Horner's rule in 128-bit
-// integers,
+// accumulators to integers, combines them in 64-bit integers,
 //
 //     T = sum_d D_d 256^(8 - d),   y u = T 2^-64 2^(er - 1021) 2^(ec - 1021),
 //
@@ -32,7 +33,7 @@
 // 2^-50 |y|max |u|max.  No FP64 arithmetic.
 //
 // Layout in shared memory (what the MMA reads): K-major, 128-byte swizzle:
-// rows of 64 bf16 (128 B) whose 16-byte chunks are permuted by XOR with the
+// rows of 64 fp16 (128 B) whose 16-byte chunks are permuted by XOR with the
 // row index mod 8, 8-row atoms of 1024 B; the two 64-wide halves of K are
 // stored one after the other.  The window task writes U's digits in exactly
 // this layout ([output half][K half][slice][column][128 B]), so one bulk
@@ -40,14 +41,17 @@
 // digits are generated by the CTA's threads.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <string.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 
 namespace gbr {
 namespace oz {
 
-constexpr long long OZ_BIAS = 0x808080808080ll;  // 128 in each of the six low digit positions
+constexpr long long OZ_BIAS = 0x80808080808080ll;  // 128 in each of the seven digit positions
 
 // G = V + OZ_BIAS for the entry x of a row (column) with exponent field emax.
 // Entries below the normal range count as zero.  Integer work only.
@@ -67,20 +71,25 @@ __host__ __device__ __forceinline__ long long oz_balanced(double x, int emax) {
     return F + OZ_BIAS;
 }
 
-// Digit p (1..7) of G = (hi:lo) as an exact float.  For p >= 2 the byte is
-// placed in the significand of 1.5 * 2^23 by a byte permute.
+// Digit P (1..7) of G0 (low half) and of G1 (high half) as two fp16 values:
+// 0x6400 | v is the fp16 number 1024 + v for v = digit + 128 in [0, 256].
 template <int P>
-__device__ __forceinline__ float oz_digit(unsigned lo, unsigned hi) {
-    if (P == 1) return __int_as_float(0x4B400000 + ((int)hi >> 16)) - 12582912.0f;
-    const unsigned src = P <= 3 ? hi : lo;
-    constexpr unsigned sel = 0x7640u | (unsigned)(P <= 3 ? 3 - P : 7 - P);
-    return __uint_as_float(__byte_perm(src, 0x4B400000u, sel)) - 12583040.0f;
-}
-
-// Two floats holding small integers -> one bf16x2 word (exact: at most 8
-// significant bits, so the low 16 bits of each float are zero).
-__device__ __forceinline__ unsigned pack_bf16x2(float lo, float hi) {
-    return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
+__device__ __forceinline__ unsigned oz_digits2(long long G0, long long G1) {
+    const unsigned lo0 = (unsigned)G0, hi0 = (unsigned)(G0 >> 32);
+    const unsigned lo1 = (unsigned)G1, hi1 = (unsigned)(G1 >> 32);
+    unsigned v;
+    if (P == 1) {
+        v = __byte_perm(hi0, hi1, 0x7632) | 0x64006400u;
+    } else {
+        constexpr unsigned b = (unsigned)(P <= 3 ? 3 - P : 7 - P);
+        v = (__byte_perm(P <= 3 ? hi0 : lo0, P <= 3 ? hi1 : lo1, 0x4400u + 0x1111u * b) & 0x00ff00ffu) |
+            0x64006400u;
+    }
+    __half2 h;
+    memcpy(&h, &v, 4);
+    h = __hadd2(h, __half2half2(__ushort_as_half(0xE480)));  // - 1152
+    memcpy(&v, &h, 4);
+    return v;
 }
 
 // Byte offset of the 16-byte chunk c (0..7) of row r in a 128-byte-swizzled
@@ -88,14 +97,14 @@ __device__ __forceinline__ unsigned pack_bf16x2(float lo, float hi) {
 __host__ __device__ constexpr int sw128(int r, int c) { return r * 128 + ((c ^ (r & 7)) << 4); }
 
 // The seven accumulators (FP32 bit patterns, diagonals 2..8) of one output ->
-// y u, given the exponent fields of its row (er) and column (ec).  The
-// accumulators hold exact integers; T = sum_d D_d 256^(8 - d) (|T| < 2^74) is
-// formed in 128-bit integers and rounded once to the nearest double: |T| is
-// shifted right by 0, 7 or 11 bits so that it fits 63 bits with at least 56
-// significant bits whenever bits are dropped, the dropped bits are kept as a
-// sticky bit in bit 0, and the 64-bit integer is converted with
-// round-to-nearest-even.  Results below the normal range flush to zero.
-__device__ __forceinline__ double oz_combine(const unsigned (&a)[7], int er, int ec) {
+// y u, given the exponent fields of its row (er) and column (ec), for any
+// exponents: T = sum_d D_d 256^(8 - d) (|T| < 2^74) is formed in 128-bit
+// integers and rounded once to the nearest double.  |T| is shifted right by 0,
+// 7 or 11 bits so that it fits 63 bits with at least 56 significant bits
+// whenever bits are dropped, the dropped bits are kept as a sticky bit in bit
+// 0, and the 64-bit integer is converted with round-to-nearest-even.  Results
+// below the normal range flush to zero.
+__device__ __forceinline__ double oz_combine_any(const unsigned (&a)[7], int er, int ec) {
     if (er == 0 || ec == 0) return 0.0;
     int D[7];
 #pragma unroll
@@ -126,6 +135,33 @@ __device__ __forceinline__ double oz_combine(const unsigned (&a)[7], int er, int
     else bits += (long long)xe << 52;
     if (neg) bits |= (long long)(1ull << 63);
     return __longlong_as_double(bits);
+}
+
+// Whether oz_combine serves the exponent fields (a result far from both ends
+// of the range, or zero).
+__device__ __forceinline__ bool oz_plain(int er, int ec) {
+    return er == 0 || ec == 0 || (unsigned)(er + ec - 1300) <= 1600u;
+}
+// The same for such exponents, in 64-bit integers: T = H 2^24 + L with |H| < 2^46, |L| < 2^40.  A
+// small T is converted as it is; otherwise 7 bits of L are dropped (rounding
+// towards minus infinity) and kept as a sticky bit in bit 0 of a number of at
+// least 55 bits, so that the one rounding of the conversion is that of T.
+// The epilogue is bound by its integer instructions: this takes about 30 of
+// them where the 128-bit form takes about 80.  With the packed digits, a task
+// of 500 panel rows (w = 128) takes 120 us; it took 137 us.
+__device__ __forceinline__ double oz_combine(const unsigned (&a)[7], int er, int ec) {
+    int D[7];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) D[j] = __float2int_rn(__uint_as_float(a[j]));  // exact
+    const long long H = (long long)(D[0] * 256 + D[1]) * 65536 + (D[2] * 256 + D[3]);
+    const long long L = (long long)D[4] * 65536 + ((long long)D[5] * 256 + D[6]);
+    const bool small = (unsigned)((int)(H >> 32) + 64) < 128u;  // |H| <= 2^38
+    const long long t = small ? (H << 24) + L
+                              : (((H << 17) + (L >> 7)) | (long long)(((unsigned)L & 127u) != 0u));
+    const double d = __ll2double_rn(t);
+    if (t == 0 || er == 0 || ec == 0) return 0.0;
+    const int xe = er + ec - 2106 + (small ? 0 : 7);
+    return __hiloint2double(__double2hiint(d) + (int)((unsigned)xe << 20), __double2loint(d));
 }
 
 // ---------------------------------------------------------------------------
@@ -203,12 +239,12 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024u >> 4) << 32) |
            (1ull << 46) | (2ull << 61);
 }
-// Instruction descriptor: bf16 x bf16 -> f32, both K-major, M = 128, N given.
+// Instruction descriptor: fp16 x fp16 -> f32, both K-major, M = 128, N given.
 constexpr uint32_t TC_M = 128, TC_N = 64;
 __host__ __device__ constexpr uint32_t idesc(uint32_t N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((TC_M >> 4) << 24);
+    return (1u << 4) | ((N >> 3) << 17) | ((TC_M >> 4) << 24);
 }
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id,
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id,
                                          uint32_t accum) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -269,7 +305,7 @@ __device__ __forceinline__ void issue_slice(int p, uint32_t a_addr, uint32_t b_a
             const uint32_t off = (uint32_t)(s & 3) * 32u;  // K step of 16 within the 128 B row
             const uint32_t ka = a_addr + (uint32_t)(s >> 2) * (uint32_t)A_KH + off;
             const uint32_t kb = bq + (uint32_t)(s >> 2) * (uint32_t)B_KH + off;
-            mma_bf16(d, sdesc(ka), sdesc(kb), id, (p == 1 && s == 0) ? 0u : 1u);
+            mma_f16(d, sdesc(ka), sdesc(kb), id, (p == 1 && s == 0) ? 0u : 1u);
         }
     }
 }
@@ -283,11 +319,7 @@ __device__ __forceinline__ void put_slice(const long long (&G)[4][8], unsigned c
     for (int i = 0; i < 4; ++i) {
         unsigned wv[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const long long g0 = G[i][2 * t], g1 = G[i][2 * t + 1];
-            wv[t] = pack_bf16x2(oz_digit<P>((unsigned)g0, (unsigned)(g0 >> 32)),
-                                oz_digit<P>((unsigned)g1, (unsigned)(g1 >> 32)));
-        }
+        for (int t = 0; t < 4; ++t) wv[t] = oz_digits2<P>(G[i][2 * t], G[i][2 * t + 1]);
         const int c16 = cq + 4 * i;
         *reinterpret_cast<uint4*>(As + (c16 >> 3) * A_KH + sw128(m, c16 & 7)) =
             make_uint4(wv[0], wv[1], wv[2], wv[3]);
@@ -517,32 +549,43 @@ static __device__ __noinline__ bool update_tile_tc(double* base, long long rs, l
             }
             // 4. epilogue: each thread one row (TMEM lane), 2 columns at a time
             const int hc = (halves == 2) ? h : 0;
+            auto epilogue = [&](auto ANY) {
 #pragma unroll 1
-            for (int c2 = 0; c2 < 8; ++c2) {
-                const int col0 = 16 * cc + 2 * c2;
-                unsigned v[NACC][2];
+                for (int c2 = 0; c2 < 8; ++c2) {
+                    const int col0 = 16 * cc + 2 * c2;
+                    unsigned v[NACC][2];
 #pragma unroll
-                for (int j = 0; j < NACC; ++j)
-                    tmem_ld2(tmem + ((uint32_t)(32 * lq) << 16) + 64u * j + (uint32_t)col0, v[j]);
-                tmem_wait_ld();
-                if (ok && r_out < pr) {
+                    for (int j = 0; j < NACC; ++j)
+                        tmem_ld2(tmem + ((uint32_t)(32 * lq) << 16) + 64u * j + (uint32_t)col0, v[j]);
+                    tmem_wait_ld();
+                    if (ok && r_out < pr) {
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const int n = h * (int)TC_N + col0 + c;
-                        if (n < w) {
-                            unsigned a[NACC];
+                        for (int c = 0; c < 2; ++c) {
+                            const int n = h * (int)TC_N + col0 + c;
+                            if (n < w) {
+                                unsigned a[NACC];
 #pragma unroll
-                            for (int j = 0; j < NACC; ++j) a[j] = v[j][c];
-                            const double y = oz_combine(a, er, cexp[hc * TC_N + col0 + c]);
-                            if (ks == 1)
-                                stg[stg_idx(r_out, col0 + c)] = y;
-                            else
-                                __stcg(&base[(long long)(y0 + p0 + r_out) * rs + (long long)n * ks],
-                                       y);
+                                for (int j = 0; j < NACC; ++j) a[j] = v[j][c];
+                                const int ec = cexp[hc * TC_N + col0 + c];
+                                const double y = decltype(ANY)::value ? oz_combine_any(a, er, ec)
+                                                                      : oz_combine(a, er, ec);
+                                if (ks == 1)
+                                    stg[stg_idx(r_out, col0 + c)] = y;
+                                else
+                                    __stcg(&base[(long long)(y0 + p0 + r_out) * rs + (long long)n * ks],
+                                           y);
+                            }
                         }
                     }
                 }
-            }
+            };
+            // (columns at or beyond w have exponent 0)
+            bool plain = true;
+            for (int c = 0; c < 16; ++c) plain = plain && oz_plain(er, cexp[hc * TC_N + 16 * cc + c]);
+            if (__all_sync(0xffffffffu, plain))
+                epilogue(std::false_type{});
+            else
+                epilogue(std::true_type{});
             if (ks == 1) {
                 // left panel: the staged outputs go out as contiguous row segments
                 if (__syncthreads_or(!ok)) return false;

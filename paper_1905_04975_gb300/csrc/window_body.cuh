@@ -28,7 +28,6 @@
 #include "ozaki.cuh"
 #include "seeded.cuh"
 
-#include <cuda_bf16.h>
 #include <float.h>
 
 #include <type_traits>
@@ -442,7 +441,7 @@ constexpr int T_11 = 0, T_3 = 1, T_22 = 2;
 
 // Writes U's digit slices for the split-precision updates (ozaki.cuh): the
 // balanced base-256 digits of every entry relative to the largest exponent of
-// its column, as bf16, in the tensor cores' 128-byte-swizzled K-major layout
+// its column, as fp16, in the tensor cores' 128-byte-swizzled K-major layout
 // [output half][K half][slice][column n mod 64][128 B] (U(k, n) is entry k of
 // column n), then one int exponent per column.  Columns/rows beyond w are
 // zero.
@@ -479,9 +478,8 @@ __device__ __forceinline__ void write_u_slices(const double* U, int w, unsigned 
                              (size_t)((c ^ (n & 7)) << 4);
         unsigned wv[4];
 #define GBR_PUT_SLICE(P)                                                                   \
-        _Pragma("unroll") for (int t = 0; t < 4; ++t) wv[t] = oz::pack_bf16x2(             \
-            oz::oz_digit<P>((unsigned)G[2 * t], (unsigned)(G[2 * t] >> 32)),                 \
-            oz::oz_digit<P>((unsigned)G[2 * t + 1], (unsigned)(G[2 * t + 1] >> 32)));       \
+        _Pragma("unroll") for (int t = 0; t < 4; ++t) wv[t] =                                  \
+            oz::oz_digits2<P>(G[2 * t], G[2 * t + 1]);                                         \
         *reinterpret_cast<uint4*>(dst + (size_t)((P) - 1) * 64 * 128) =                    \
             make_uint4(wv[0], wv[1], wv[2], wv[3]);
         GBR_PUT_SLICE(1) GBR_PUT_SLICE(2) GBR_PUT_SLICE(3) GBR_PUT_SLICE(4) GBR_PUT_SLICE(5)
