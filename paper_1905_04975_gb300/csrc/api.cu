@@ -3,6 +3,8 @@
 // or one window/update launch pair per window), re-plan after rejected swaps.
 #include "host.h"
 
+#include <stdlib.h>
+
 #include <algorithm>
 #include <chrono>
 #include <climits>
@@ -132,7 +134,7 @@ static int read_err(const SchedLaunch& L, cudaStream_t s, int* acc) {
 // alternate between the pool slots pl.slot[0] and pl.slot[1].
 int run_pass_persistent(const std::vector<Window>& wins, const PassLaunch& pl, const gbr_opts& o,
                         long long* ntasks_out, double* ms_out, long long* launches_out,
-                        SchedInfo* info, cudaStream_t st) {
+                        SchedInfo* info, cudaStream_t st, const std::function<int()>& tail) {
     std::vector<Window> all = wins;
     pipeline_order(pl.inst.n, all);
     const std::vector<size_t> cuts = chunk_cuts(all.size(), o);
@@ -188,7 +190,7 @@ int run_pass_persistent(const std::vector<Window>& wins, const PassLaunch& pl, c
                     void* p = nullptr;
                     return pool_get(slot, bytes, &p) ? nullptr : p;
                 },
-                &L[b], &inf, up);
+                &L[b], &inf, up, up != st);
             if (rc) return rc;
             if (pl.mode >= 0) L[b].P.mode = pl.mode;
             tot.tasks += inf.tasks;
@@ -197,7 +199,7 @@ int run_pass_persistent(const std::vector<Window>& wins, const PassLaunch& pl, c
             tot.graph_ms += inf.graph_ms;
             tot.order_ms += inf.order_ms;
             if (c == 0 && o.timing) GBR_CK(cudaEventRecord(ev.e[0], st), "event");
-            rc = sched_enqueue(L[b], st);
+            rc = sched_enqueue(L[b], st, nullptr, true);
             if (rc) return rc;
             if (nch > 1) GBR_CK(cudaEventRecord(ev.e[2 + b], st), "event");
             *ntasks_out += L[b].P.ntasks;
@@ -210,6 +212,13 @@ int run_pass_persistent(const std::vector<Window>& wins, const PassLaunch& pl, c
         return rc_loop;
     }
     if (o.timing) GBR_CK(cudaEventRecord(ev.e[1], st), "event");
+    if (tail) {
+        const int rct = tail();
+        if (rct) {
+            (void)cudaStreamSynchronize(st);
+            return rct;
+        }
+    }
     for (int c = std::max(0, nch - 2); c < nch; ++c) {
         int rce = read_err(L[c & 1], st, &h_err);
         if (rce) return rce;
@@ -238,14 +247,14 @@ int run_pass_persistent(const std::vector<Window>& wins, const PassLaunch& pl, c
 static int run_persistent(int n, const std::vector<Window>& wins, double* S, int ldS, double* Q,
                           int ldQ, uint8_t* d_sel, DevCounters* d_ctr, const gbr_opts& o,
                           long long* ntasks_out, double* ms_out, long long* launches_out,
-                          cudaStream_t st) {
+                          cudaStream_t st, const std::function<int()>& tail) {
     PassLaunch pl{};
     pl.inst = Inst{S, Q, d_sel, d_ctr, n, ldS, ldQ, 0};
     pl.cm = cost_model(o);
     pl.slot[0] = POOL_SCHED;
     pl.slot[1] = POOL_SCHED_ALT;
     pl.timeout_msg = "persistent scheduler: a task waited longer than wait_limit_ms";
-    return run_pass_persistent(wins, pl, o, ntasks_out, ms_out, launches_out, &g_last_sched, st);
+    return run_pass_persistent(wins, pl, o, ntasks_out, ms_out, launches_out, &g_last_sched, st, tail);
 }
 
 // ---------------------------------------------------------------------------
@@ -286,7 +295,39 @@ static constexpr ScratchLayout scratch_layout(size_t n) {
                              (size_t)WMAX * WMAX * sizeof(double)};
 }
 
-static int reorder_device_at(char* b, int n, double* S, int ldS, double* Q, int ldQ,
+// Host staging of a call, under the lock like the device pool: page-locked,
+// so that the device copies to it without a host-side wait per copy.  Plain
+// memory registered with CUDA: after a device reset it is still memory, and
+// copies to it are only slower.  Grow-only; gbr_release gives it back.
+struct HostStage {
+    char* p = nullptr;
+    size_t bytes = 0;
+    bool registered = false;
+};
+static HostStage g_stage;
+static void stage_free() {
+    if (g_stage.registered && cudaHostUnregister(g_stage.p) != cudaSuccess) (void)cudaGetLastError();
+    free(g_stage.p);
+    g_stage = HostStage{};
+}
+static int stage_get(size_t bytes, char** out) {
+    if (g_stage.bytes < bytes) {
+        stage_free();
+        const size_t grow = (bytes + bytes / 4 + 65535) & ~(size_t)65535;
+        g_stage.p = (char*)aligned_alloc(65536, grow);
+        if (!g_stage.p) return GBR_ERR_NOMEM;
+        g_stage.bytes = grow;
+        g_stage.registered = cudaHostRegister(g_stage.p, grow, cudaHostRegisterPortable) == cudaSuccess;
+        if (!g_stage.registered) (void)cudaGetLastError();  // a slower copy, nothing else
+    }
+    *out = g_stage.p;
+    return 0;
+}
+
+// b: device scratch, stage: host memory, both laid out by scratch_layout (the
+// host one without U).  On an error the stream is drained before it returns,
+// so that no copy from or to the staging memory is under way any more.
+static int reorder_device_at(char* b, char* stage, int n, double* S, int ldS, double* Q, int ldQ,
                              const int* select, double* eig_re, double* eig_im, int* m_out,
                              const gbr_opts& o, gbr_stats* stats, cudaStream_t st);
 
@@ -294,13 +335,18 @@ static int reorder_device(int n, double* S, int ldS, double* Q, int ldQ, const i
                           double* eig_re, double* eig_im, int* m_out, const gbr_opts& o,
                           gbr_stats* stats, cudaStream_t st) {
     void* base = nullptr;
+    char* stage = nullptr;
     int rc = pool_get(POOL_SCRATCH, scratch_layout(n).total, &base);
     if (rc) return rc;
-    return reorder_device_at((char*)base, n, S, ldS, Q, ldQ, select, eig_re, eig_im, m_out, o,
-                             stats, st);
+    rc = stage_get(scratch_layout(n).off_u, &stage);
+    if (rc) return rc;
+    rc = reorder_device_at((char*)base, stage, n, S, ldS, Q, ldQ, select, eig_re, eig_im, m_out, o,
+                           stats, st);
+    if (rc < 0) (void)cudaStreamSynchronize(st);
+    return rc;
 }
 
-static int reorder_device_at(char* b, int n, double* S, int ldS, double* Q, int ldQ,
+static int reorder_device_at(char* b, char* stage, int n, double* S, int ldS, double* Q, int ldQ,
                              const int* select, double* eig_re, double* eig_im, int* m_out,
                              const gbr_opts& o, gbr_stats* stats, cudaStream_t st) {
     const ScratchLayout L = scratch_layout(n);
@@ -311,21 +357,25 @@ static int reorder_device_at(char* b, int n, double* S, int ldS, double* Q, int 
     uint8_t* d_sel = (uint8_t*)(b + off_sel);
     double* d_eig = (double*)(b + off_eig);
     double* d_u = (double*)(b + off_u);
+    DevCounters& h_ctr = *(DevCounters*)(stage + off_ctr);
+    uint8_t* const sub = (uint8_t*)(stage + off_sub);
+    uint8_t* const sel = (uint8_t*)(stage + off_sel);
+    const double* const h_eig = (const double*)(stage + off_eig);
+    const bool want_eig = eig_re || eig_im;
 
-    DevCounters h_ctr{0, 0, INT_MAX, 0, 0};
+    h_ctr = DevCounters{0, 0, INT_MAX, 0, 0};
     GBR_CK(cudaMemcpyAsync(d_ctr, &h_ctr, sizeof h_ctr, cudaMemcpyHostToDevice, st), "H2D counters");
     NvtxRange nv_call("gbr_reorder");
-    if (o.validate) GBR_CK(launch_validate(n, S, ldS, d_ctr, st), "validate kernel");
-    GBR_CK(launch_subdiag(n, S, ldS, d_sub, st), "subdiag kernel");
-    std::vector<uint8_t> sub(n), sel(n);
-    GBR_CK(cudaMemcpyAsync(sub.data(), d_sub, n, cudaMemcpyDeviceToHost, st), "D2H subdiag");
-    GBR_CK(cudaMemcpyAsync(&h_ctr, d_ctr, sizeof h_ctr, cudaMemcpyDeviceToHost, st), "D2H counters");
+    if (o.validate) GBR_CK(launch_validate(n, S, ldS, d_ctr, st, d_sub), "validate kernel");
+    else GBR_CK(launch_subdiag(n, S, ldS, d_sub, st), "subdiag kernel");
+    // counters and 2x2 pattern in one copy
+    GBR_CK(cudaMemcpyAsync(stage, b, off_sub + (size_t)n, cudaMemcpyDeviceToHost, st), "D2H pattern");
     GBR_CK(cudaStreamSynchronize(st), "sync");
     if (h_ctr.bad_column != INT_MAX) return -2;
 
     // selection per position; a 2x2 block is selected if either row is
-    const int msel = selection_positions(n, sub.data(), select, sel.data());
-    GBR_CK(cudaMemcpyAsync(d_sel, sel.data(), n, cudaMemcpyHostToDevice, st), "H2D selection");
+    const int msel = selection_positions(n, sub, select, sel);
+    GBR_CK(cudaMemcpyAsync(d_sel, sel, n, cudaMemcpyHostToDevice, st), "H2D selection");
 
     // optional per-kernel event timing: one event pair per launch, read at the end
     struct Events {
@@ -344,10 +394,19 @@ static int reorder_device_at(char* b, int n, double* S, int ldS, double* Q, int 
         v.push_back(ev);
         return cudaEventRecord(ev, st);
     };
-    long long launches = o.validate ? 2 : 1;
+    long long launches = 1;
 
     PlanState ps;
-    init_state(ps, n, sub.data(), sel.data());
+    init_state(ps, n, sub, sel);
+    // after a pass: eigenvalues (those of the result if nothing was rejected)
+    // and counters, in one copy that the pass's own wait covers
+    auto fetch = [&]() -> int {
+        if (want_eig) GBR_CK(launch_eigs(n, S, ldS, d_eig, d_eig + n, st), "eigenvalue kernel");
+        const size_t bytes = want_eig ? off_eig + 2 * sizeof(double) * (size_t)n : sizeof(DevCounters);
+        GBR_CK(cudaMemcpyAsync(stage, b, bytes, cudaMemcpyDeviceToHost, st), "D2H counters");
+        return 0;
+    };
+    bool fetched = false;
     long long nwin = 0;
     int nchains = 0;
     double flops = 0.0;
@@ -363,8 +422,9 @@ static int reorder_device_at(char* b, int n, double* S, int ldS, double* Q, int 
         if (win.empty()) break;
         if (o.sched == GBR_SCHED_PERSISTENT) {
             int rcs = run_persistent(n, win, S, ldS, Q, ldQ, d_sel, d_ctr, o, &ntasks, &ms_sched,
-                                     &launches, st);
+                                     &launches, st, fetch);
             if (rcs) return rcs;
+            fetched = true;
             flops += update_flops(n, win, Q != nullptr);
         } else
         {
@@ -383,32 +443,30 @@ static int reorder_device_at(char* b, int n, double* S, int ldS, double* Q, int 
           }
         }
         nwin += (long long)win.size();
-        GBR_CK(cudaMemcpyAsync(&h_ctr, d_ctr, sizeof h_ctr, cudaMemcpyDeviceToHost, st), "D2H counters");
-        GBR_CK(cudaStreamSynchronize(st), "sync");
+        if (!fetched) {
+            GBR_CK(cudaMemcpyAsync(&h_ctr, d_ctr, sizeof h_ctr, cudaMemcpyDeviceToHost, st), "D2H counters");
+            GBR_CK(cudaStreamSynchronize(st), "sync");
+        }
         if (h_ctr.rejected == seen_rej) break;  // the simulated plan was exact
         if (o.on_reject == GBR_ON_REJECT_ABORT) break;  // stopped at the first rejection
         seen_rej = h_ctr.rejected;
         // re-plan from the device state: stuck blocks are barriers now
         GBR_CK(launch_subdiag(n, S, ldS, d_sub, st), "subdiag kernel");
-        GBR_CK(cudaMemcpyAsync(sub.data(), d_sub, n, cudaMemcpyDeviceToHost, st), "D2H subdiag");
-        GBR_CK(cudaMemcpyAsync(sel.data(), d_sel, n, cudaMemcpyDeviceToHost, st), "D2H selection");
+        GBR_CK(cudaMemcpyAsync(sub, d_sub, n, cudaMemcpyDeviceToHost, st), "D2H subdiag");
+        GBR_CK(cudaMemcpyAsync(sel, d_sel, n, cudaMemcpyDeviceToHost, st), "D2H selection");
         GBR_CK(cudaStreamSynchronize(st), "sync");
-        init_state(ps, n, sub.data(), sel.data());
+        init_state(ps, n, sub, sel);
         launches += 1;
     }
 
-    if (eig_re || eig_im) {
-        GBR_CK(launch_eigs(n, S, ldS, d_eig, d_eig + n, st), "eigenvalue kernel");
-        if (eig_re)
-            GBR_CK(cudaMemcpyAsync(eig_re, d_eig, n * sizeof(double), cudaMemcpyDeviceToHost, st),
-                   "D2H eig_re");
-        if (eig_im)
-            GBR_CK(cudaMemcpyAsync(eig_im, d_eig + n, n * sizeof(double), cudaMemcpyDeviceToHost, st),
-                   "D2H eig_im");
+    if (!fetched) {
+        const int rcf = fetch();
+        if (rcf) return rcf;
+        GBR_CK(cudaStreamSynchronize(st), "sync");
     }
-    if (eig_re || eig_im) launches += 1;
-    GBR_CK(cudaMemcpyAsync(&h_ctr, d_ctr, sizeof h_ctr, cudaMemcpyDeviceToHost, st), "D2H counters");
-    GBR_CK(cudaStreamSynchronize(st), "sync");
+    if (eig_re) memcpy(eig_re, h_eig, n * sizeof(double));
+    if (eig_im) memcpy(eig_im, h_eig + n, n * sizeof(double));
+    if (want_eig) launches += 1;
     double msw = 0.0, msu = 0.0;
     for (size_t i = 0; i + 1 < evw.size(); i += 2) {
         float t = 0.f;
@@ -646,8 +704,10 @@ int gbr_reorder_noalloc(int n, double* S, int ldS, double* Q, int ldQ, const int
     char* base = nullptr;
     rc = noalloc_scratch(&base);
     if (rc) return rc;
-    rc = reorder_device_at(base, n, S, ldS, Q, ldQ, select, eig_re, eig_im, m_out, o, stats,
-                           (cudaStream_t)cuda_stream);
+    std::vector<char> stage(scratch_layout(n).off_u);  // nothing is page-locked here either
+    rc = reorder_device_at(base, stage.data(), n, S, ldS, Q, ldQ, select, eig_re, eig_im, m_out, o,
+                           stats, (cudaStream_t)cuda_stream);
+    if (rc < 0) (void)cudaStreamSynchronize((cudaStream_t)cuda_stream);
     if (stats)
         stats->ms_total =
             std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -880,6 +940,7 @@ void gbr_release(void) {
         cudaStreamDestroy(g_side[dev]);
         g_side[dev] = nullptr;
     }
+    stage_free();
 }
 
 int gbr_version(void) { return 100; }

@@ -152,7 +152,8 @@ struct SrvParams {
 };
 
 // Launchers (each .cu file owns its kernels).
-cudaError_t launch_validate(int n, const double* S, int ldS, DevCounters* ctr, cudaStream_t st);
+cudaError_t launch_validate(int n, const double* S, int ldS, DevCounters* ctr, cudaStream_t st,
+                            uint8_t* sub = nullptr);
 cudaError_t launch_subdiag(int n, const double* S, int ldS, uint8_t* sub, cudaStream_t st);
 cudaError_t launch_eigs(int n, const double* S, int ldS, double* wr, double* wi, cudaStream_t st);
 cudaError_t launch_window(int n, const Window& w, double* S, int ldS, uint8_t* sel, double* U,

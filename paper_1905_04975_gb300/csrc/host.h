@@ -9,6 +9,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <functional>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -163,19 +164,24 @@ struct SchedLaunch {
     int* ctl = nullptr;               // head, err (and spare words), 256 bytes
     size_t trace_bytes = 0;
     std::vector<SchedTask> tq;        // host copy of the queue (trace decoding)
+    std::unique_ptr<char[]> image;    // host source of the upload (kept until it has run)
 };
 
 // Plans the task graph of all instances, orders it for `grid` CTAs, and
 // uploads it into device memory obtained from alloc(bytes) (which must
-// return 256-byte aligned memory that outlives the launches, or null).
+// return 256-byte aligned memory that outlives the launches, or null).  The
+// upload is one copy on st; with wait it has finished on return (needed when
+// the launch goes to another stream).
 int sched_prepare(std::vector<InstPlan>& plans, const gbr_opts& o, const CostModel& cm, int grid,
                   const std::function<void*(size_t)>& alloc, SchedLaunch* L, SchedInfo* info,
-                  cudaStream_t st);
+                  cudaStream_t st, bool wait = true);
 // Enqueues one launch: dependency counters restored, control words reset,
 // then pre(st) if given (it may set *P.err to stop the launch early), then
-// the kernel.  Only stream operations: capturable into a CUDA graph.
+// the kernel.  Only stream operations: capturable into a CUDA graph.  fresh:
+// the image's first launch after its upload, which brought the counters and
+// control words.
 int sched_enqueue(const SchedLaunch& L, cudaStream_t st,
-                  const std::function<int(cudaStream_t)>& pre = nullptr);
+                  const std::function<int(cudaStream_t)>& pre = nullptr, bool fresh = false);
 // Keeps the per-task timeline of a finished traced launch (opts.timing = 2)
 // for gbr_last_trace.
 int store_trace(const SchedLaunch& L);
@@ -194,8 +200,10 @@ struct PassLaunch {
 };
 // Adds the tasks, the launches and (with opts.timing) the launches' device
 // time to the outputs; *info receives the chunks' planning figures summed.
+// tail (nullable) enqueues more work on st before the stream is waited for.
 int run_pass_persistent(const std::vector<Window>& wins, const PassLaunch& pl, const gbr_opts& o,
                         long long* ntasks_out, double* ms_out, long long* launches_out,
-                        SchedInfo* info, cudaStream_t st);
+                        SchedInfo* info, cudaStream_t st,
+                        const std::function<int()>& tail = nullptr);
 
 }  // namespace gbr

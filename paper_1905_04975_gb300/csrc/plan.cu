@@ -14,8 +14,11 @@
 // the device (stuck blocks then act as barriers) until nothing can move.
 #include "host.h"
 
+#include <string.h>
+
 #include <algorithm>
 #include <chrono>
+#include <new>
 #include <cstdio>
 #include <cstring>
 #include <queue>
@@ -328,7 +331,9 @@ void build_graph(int n, const std::vector<Window>& wins, bool withQ, const CostM
         }
     };
     const int nqb = (n + FAR - 1) / FAR;
-    const int NT = std::max(1, std::min(threads, nc));
+    // a thread for every 512 tasks at most: starting one takes about as long
+    // as the search for a few hundred tasks
+    const int NT = std::max(1, std::min({threads, nc, (int)(T.size() / 512)}));
     std::vector<std::vector<std::pair<int, int>>> tedges(NT);
     auto worker = [&](int k) {
         std::vector<std::pair<int, int>>& out = tedges[k];
@@ -530,7 +535,7 @@ void queue_order(const TaskGraph& G, int P, std::vector<int>& order, double* cp_
 // ---------------------------------------------------------------------------
 int sched_prepare(std::vector<InstPlan>& plans, const gbr_opts& o, const CostModel& cm, int grid,
                   const std::function<void*(size_t)>& alloc, SchedLaunch* L, SchedInfo* info,
-                  cudaStream_t st) {
+                  cudaStream_t st, bool wait) {
     const bool ozaki = (o.precision == GBR_PREC_OZAKI);
     const size_t ni = plans.size();
     auto th0 = std::chrono::steady_clock::now();
@@ -602,24 +607,6 @@ int sched_prepare(std::vector<InstPlan>& plans, const gbr_opts& o, const CostMod
         info->graph_ms = std::chrono::duration<double, std::milli>(th1 - th0).count();
         info->order_ms = std::chrono::duration<double, std::milli>(th2 - th1).count();
     }
-    std::vector<int> pos(nt);
-    for (int q = 0; q < nt; ++q) pos[order[q]] = q;
-    std::vector<SchedTask> tq(nt);
-    std::vector<int> deps(nt), soff(nt + 1, 0), succ(M.succ.size());
-    for (int q = 0; q < nt; ++q) {
-        const HostTask& h = M.t[order[q]];
-        tq[q] = SchedTask{h.kind, h.win, h.y0, h.rows};
-        deps[q] = M.ndeps[order[q]];
-        soff[q + 1] = soff[q] + (M.soff[order[q] + 1] - M.soff[order[q]]);
-    }
-    for (int q = 0; q < nt; ++q) {
-        int t = order[q], o2 = soff[q];
-        for (int i = M.soff[t]; i < M.soff[t + 1]; ++i) succ[o2++] = pos[M.succ[i]];
-    }
-    if ((o.inject & GBR_INJECT_STALL) && nt > 1) deps[nt - 1] += 1;  // a predecessor that never ends
-    std::vector<Inst> itab(ni);
-    for (size_t i = 0; i < ni; ++i) itab[i] = plans[i].d;
-
     // device image: inst | tasks | wins | deps | deps_init | soff | succ | ctl | trace | U slices
     // | split-precision scratch | U pool
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
@@ -628,7 +615,7 @@ int sched_prepare(std::vector<InstPlan>& plans, const gbr_opts& o, const CostMod
     const size_t b_wins = al(sizeof(Window) * std::max<size_t>(1, wins.size()));
     const size_t b_deps = al(sizeof(int) * std::max(1, nt));
     const size_t b_soff = al(sizeof(int) * (nt + 1));
-    const size_t b_succ = al(sizeof(int) * std::max<size_t>(1, succ.size()));
+    const size_t b_succ = al(sizeof(int) * std::max<size_t>(1, M.succ.size()));
     const size_t b_ctl = 256;
     const size_t b_tr = (o.timing >= 2) ? al(sizeof(unsigned long long) * 4 * std::max(1, nt)) : 0;
     // digit slices per window: one U, or UQ and UZ for a generalized instance
@@ -654,6 +641,7 @@ int sched_prepare(std::vector<InstPlan>& plans, const gbr_opts& o, const CostMod
                          b_us + b_ws + b_wscr + b_u;
     char* p = (char*)alloc(total);
     if (!p) return GBR_ERR_NOMEM;
+    char* const base = p;
     Inst* d_inst = (Inst*)p; p += b_inst;
     SchedTask* d_tasks = (SchedTask*)p; p += b_tasks;
     Window* d_wins = (Window*)p; p += b_wins;
@@ -667,17 +655,36 @@ int sched_prepare(std::vector<InstPlan>& plans, const gbr_opts& o, const CostMod
     int* d_ws = b_ws ? (int*)p : nullptr; p += b_ws;
     double* d_wscr = b_wscr ? (double*)p : nullptr; p += b_wscr;
     double* d_u = (double*)p;
-    GBR_CK(cudaMemcpyAsync(d_inst, itab.data(), sizeof(Inst) * ni, cudaMemcpyHostToDevice, st), "H2D instances");
-    if (nt) {
-        GBR_CK(cudaMemcpyAsync(d_tasks, tq.data(), sizeof(SchedTask) * nt, cudaMemcpyHostToDevice, st), "H2D tasks");
-        GBR_CK(cudaMemcpyAsync(d_deps0, deps.data(), sizeof(int) * nt, cudaMemcpyHostToDevice, st), "H2D deps");
+    // everything up to the control words is built in one host image (in the
+    // same layout) and uploaded by one copy; the counters and the control
+    // words come with it, ready for a first launch
+    const size_t b_img = b_inst + b_tasks + b_wins + 2 * b_deps + b_soff + b_succ + b_ctl;
+    L->image.reset(new (std::nothrow) char[b_img]);
+    if (!L->image) return GBR_ERR_NOMEM;
+    const auto host = [&](const void* d) { return L->image.get() + ((const char*)d - base); };
+    SchedTask* tq = (SchedTask*)host(d_tasks);
+    int* deps = (int*)host(d_deps0);
+    int* soff = (int*)host(d_soff);
+    int* succ = (int*)host(d_succ);
+    for (size_t i = 0; i < ni; ++i) ((Inst*)host(d_inst))[i] = plans[i].d;
+    std::copy(wins.begin(), wins.end(), (Window*)host(d_wins));
+    std::vector<int> pos(nt);
+    for (int q = 0; q < nt; ++q) pos[order[q]] = q;
+    soff[0] = 0;
+    for (int q = 0; q < nt; ++q) {
+        const int t = order[q];
+        const HostTask& h = M.t[t];
+        tq[q] = SchedTask{h.kind, h.win, h.y0, h.rows};
+        deps[q] = M.ndeps[t];
+        int o2 = soff[q];
+        for (int i = M.soff[t]; i < M.soff[t + 1]; ++i) succ[o2++] = pos[M.succ[i]];
+        soff[q + 1] = o2;
     }
-    if (!wins.empty())
-        GBR_CK(cudaMemcpyAsync(d_wins, wins.data(), sizeof(Window) * wins.size(), cudaMemcpyHostToDevice, st), "H2D windows");
-    GBR_CK(cudaMemcpyAsync(d_soff, soff.data(), sizeof(int) * (nt + 1), cudaMemcpyHostToDevice, st), "H2D succ offsets");
-    if (!succ.empty())
-        GBR_CK(cudaMemcpyAsync(d_succ, succ.data(), sizeof(int) * succ.size(), cudaMemcpyHostToDevice, st), "H2D succ");
-    GBR_CK(cudaStreamSynchronize(st), "sync");  // the host vectors go out of scope
+    if ((o.inject & GBR_INJECT_STALL) && nt > 1) deps[nt - 1] += 1;  // a predecessor that never ends
+    memcpy(host(d_deps), deps, sizeof(int) * nt);
+    memset(host(d_ctl), 0, b_ctl);
+    GBR_CK(cudaMemcpyAsync(base, L->image.get(), b_img, cudaMemcpyHostToDevice, st), "H2D launch image");
+    if (wait) GBR_CK(cudaStreamSynchronize(st), "sync");
 
     SchedParams& P = L->P;
     P = SchedParams{};
@@ -705,16 +712,17 @@ int sched_prepare(std::vector<InstPlan>& plans, const gbr_opts& o, const CostMod
     L->deps_init = d_deps0;
     L->ctl = d_ctl;
     L->trace_bytes = b_tr;
-    if (b_tr) L->tq.swap(tq);
-    else L->tq.clear();
+    L->tq.clear();
+    if (b_tr) L->tq.assign(tq, tq + nt);
     return 0;
 }
 
-int sched_enqueue(const SchedLaunch& L, cudaStream_t st, const std::function<int(cudaStream_t)>& pre) {
-    if (L.P.ntasks > 0)
+int sched_enqueue(const SchedLaunch& L, cudaStream_t st, const std::function<int(cudaStream_t)>& pre,
+                  bool fresh) {
+    if (L.P.ntasks > 0 && !fresh)
         GBR_CK(cudaMemcpyAsync(L.P.deps_left, L.deps_init, sizeof(int) * L.P.ntasks,
                                cudaMemcpyDeviceToDevice, st), "restore dependency counters");
-    GBR_CK(cudaMemsetAsync(L.ctl, 0, 256, st), "memset control");
+    if (!fresh) GBR_CK(cudaMemsetAsync(L.ctl, 0, 256, st), "memset control");
     if (L.trace_bytes) GBR_CK(cudaMemsetAsync(L.P.trace, 0, L.trace_bytes, st), "memset trace");
     if (pre) {
         int rc = pre(st);

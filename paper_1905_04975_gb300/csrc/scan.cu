@@ -11,9 +11,10 @@ namespace {
 
 // One warp per column: entries two or more below the diagonal must be zero;
 // a 2x2 block [[a, b], [c, d]] (c != 0) must not overlap the next block and
-// must be standardized (a == d, bc < 0).
+// must be standardized (a == d, bc < 0).  sub (nullable) receives the
+// subdiagonal pattern, as subdiag_kernel writes it.
 __global__ void validate_kernel(int n, const double* __restrict__ S, int ldS,
-                                DevCounters* __restrict__ ctr) {
+                                DevCounters* __restrict__ ctr, uint8_t* __restrict__ sub) {
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -21,6 +22,7 @@ __global__ void validate_kernel(int n, const double* __restrict__ S, int ldS,
         bool bad = false;
         const double* col = S + cm(0, j, ldS);
         for (int i = j + 2 + lane; i < n; i += 32) bad |= (col[i] != 0.0);
+        if (sub && lane == 0) sub[j] = (j + 1 < n && col[j + 1] != 0.0) ? 1 : 0;
         if (lane == 0 && j + 1 < n && col[j + 1] != 0.0) {
             double a = col[j], c = col[j + 1];
             double b = S[cm(j, j + 1, ldS)], d = S[cm(j + 1, j + 1, ldS)];
@@ -104,11 +106,12 @@ int grid_for(int n, int threads) {
 
 }  // namespace
 
-cudaError_t launch_validate(int n, const double* S, int ldS, DevCounters* ctr, cudaStream_t st) {
+cudaError_t launch_validate(int n, const double* S, int ldS, DevCounters* ctr, cudaStream_t st,
+                            uint8_t* sub) {
     if (n <= 0) return cudaSuccess;
     int warps = n < 152 * 64 ? n : 152 * 64;
     int blocks = (warps * 32 + 255) / 256;
-    validate_kernel<<<blocks, 256, 0, st>>>(n, S, ldS, ctr);
+    validate_kernel<<<blocks, 256, 0, st>>>(n, S, ldS, ctr, sub);
     return cudaGetLastError();
 }
 
