@@ -625,8 +625,8 @@ __device__ __forceinline__ int prefix_slot(const int* pre, int lo, int hi, int i
 // Named barriers of the window task's two warp groups (barrier 0 is
 // __syncthreads): PRODUCTS among the product warps, CRIT from the product
 // warps (arrive) to the transform warps (wait).
-__device__ __forceinline__ void bar_products() {
-    asm volatile("bar.sync 1, %0;" ::"n"(WIN_THREADS - 32 * WIN_TWARPS) : "memory");
+__device__ __forceinline__ void bar_products(int threads) {
+    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
 }
 __device__ __forceinline__ void bar_crit_arrive() {
     asm volatile("bar.arrive 2, %0;" ::"n"(WIN_THREADS) : "memory");
@@ -1041,13 +1041,22 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
     // transform warps load some sub-partitions' pipes more than others, so
     // the warps of the less loaded sub-partitions take more items.
     // has = the step had swaps; the barriers run either way.
+    // A small window is bound by the chains of its transforms (w = 32: 7.1K of
+    // a step's 10.3K cycles), and the longest one, on warp 0, would share its
+    // sub-partition's FP64 pipe with three product warps: there they stay
+    // away.  A large window is bound by the products and uses all of them.
+    // Measured, a whole window with and without: w = 32 173 and 176 us, w = 48
+    // 245 and 257 us, w = 64 343 and 362 us; at w = 96 it costs 3%.
+    constexpr int FEW_W = 64;
+    const bool few = w <= FEW_W;
+    const int npw = (WIN_THREADS / 32 - NTW) - (few ? WIN_THREADS / 128 - NTW / 4 : 0);  // product warps
+    const int pw = few ? ((warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 - NTW / 4 * 3 : -1) : warp - NTW;
     __shared__ int pclaim[2][4];  // by the parity of the step applied
     auto products = [&](int pp, bool has) {
         const double* Zs = Zbuf + pp * MSW * 16;
         const int* desc = swbuf + pp * MSW;
         const int m4 = tcnt2[pp][T_22], m3 = tcnt2[pp][T_3], m2 = tcnt2[pp][T_11];
         constexpr int NCL = CRIT_L - 2, NCR = CRIT_R - 2;  // item slots per swap
-        constexpr int NPW = WIN_THREADS / 32 - NTW;        // product warps
         // The items of part `ph` (t4, t3, t2 of them per size), by chunks of
         // one size, those with the most work per item first: PER items per
         // lane (one for k = 4).  The first chunk of a warp is its own; the
@@ -1064,17 +1073,17 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                 else
                     item_run2<k>(item(K, min(it, t - 1), it < t), item(K, min(it + 32, t - 1), it + 32 < t));
             };
-            for (int c = warp - NTW; c < n;) {
+            for (int c = pw; c < n;) {
                 int nx = 0;
-                if (n > NPW && lane == 0) nx = atomicAdd(&pclaim[pp][ph], 1);
+                if (n > npw && lane == 0) nx = atomicAdd(&pclaim[pp][ph], 1);
                 if (c < c4)
                     chunk(std::integral_constant<int, 4>{}, 32 * c, t4);
                 else if (c < c3)
                     chunk(std::integral_constant<int, 3>{}, 32 * per * (c - c4), t3);
                 else
                     chunk(std::integral_constant<int, 2>{}, 32 * per * (c - c3), t2);
-                if (n <= NPW) break;
-                c = NPW + __shfl_sync(0xffffffffu, nx, 0);
+                if (n <= npw) break;
+                c = npw + __shfl_sync(0xffffffffu, nx, 0);
             }
         };
         // slots of size k: first one and their number
@@ -1088,7 +1097,7 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                 const int slot = first(k) + it / NCL, d = desc[slot], j = sw_j(d), c = j + k + it % NCL;
                 return make_item<k>(Sp + poff(c) + j, 1, 0, d, Zs + slot * 16, ok && c < min(w, j + CRIT_L));
             });
-        bar_products();
+        bar_products(32 * npw);
         if (has)
             part(PER1, 1, m4 * NCR, m3 * NCR, m2 * NCR, [&](auto K, int it, bool ok) {
                 constexpr int k = decltype(K)::value;
@@ -1111,7 +1120,7 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
                      return make_item<k>(Sp + poff(j + CRIT_L + (it - pl[slot])) + j, 1, 0, d, Zs + slot * 16,
                                          ok);
                  });
-        bar_products();
+        bar_products(32 * npw);
         if (has) {
             // far right rows of S, then the rows of U, of each size
             const int s4 = ps[m4], s3 = ps[m4 + m3] - s4, s2 = ps[m4 + m3 + m2] - ps[m4 + m3];
@@ -1169,8 +1178,10 @@ __device__ __forceinline__ void window_body_t(int n, double* __restrict__ S, int
             const int ns = nsw[pi];
             if (ns > 0) transforms(pi);
             if (warp == NTW - 1 && ns > 0) prefix_sums(pi, ns);
-        } else {
+        } else if (pw >= 0) {
             products(pp, ns_prev > 0);
+        } else {
+            bar_crit_arrive();
         }
         __syncthreads();
         ns_prev = nsw[pi];
