@@ -251,6 +251,7 @@ static int run_persistent(int n, const std::vector<Window>& wins, double* S, int
     PassLaunch pl{};
     pl.inst = Inst{S, Q, d_sel, d_ctr, n, ldS, ldQ, 0};
     pl.cm = cost_model(o);
+    tile_heights(pl.cm, n, o.window, o.precision, false);
     pl.slot[0] = POOL_SCHED;
     pl.slot[1] = POOL_SCHED_ALT;
     pl.timeout_msg = "persistent scheduler: a task waited longer than wait_limit_ms";

@@ -220,6 +220,7 @@ int run_persistent_gen(int n, const std::vector<Window>& wins, double* S, int ld
     pl.cm.win_us_128 = kGenWinUs128;
     if (o.precision == GBR_PREC_OZAKI) pl.cm.tile_rate = 100000.0;
     if (o.precision == GBR_PREC_FMA) pl.cm.tile_rate = 7600.0;
+    tile_heights(pl.cm, n, o.window, o.precision, true);
     pl.slot[0] = POOL_GEN_SCHED;
     pl.slot[1] = POOL_GEN_SCHED_ALT;
     pl.mode = 1;

@@ -129,7 +129,34 @@ struct CostModel {
     double tile_rate = 6900.0;   // update flops per microsecond of one SM
     double task_us = 2.0;        // fixed cost per update task
     double lr_mats = 1.0;        // matrices a left/right tile updates (2 for (S, T))
+    int near = UPD_BM;           // rows of the tiles near a window (a divisor or multiple of UPD_BM)
+    int far_mul = 1;             // factor on far_rows(n)
 };
+
+// Tile heights of one reordering (pair: of (S, T)); the batched path and the
+// server, which fill the device with many problems, keep the defaults.
+//
+// FP64: the next window of a chain waits for a near tile of 64 rows (210 us at
+// w = 128, beside a window task of 1.3 ms).  On a small form most SMs wait
+// anyway, and tiles of 32 rows halve that; on a large one the device is full
+// and the second load of U per 64 rows costs.  Measured, ms with 64 and 32
+// rows, w = 128: n = 600 8.83 and 8.26, 1200 18.8 and 17.6, 2200 36.3 and 35.7,
+// 3000 57.0 and 56.6, 4000 96.3 and 99.0; w = 64: n = 1500 15.7 and 16.1; pairs
+// (w = 64): n = 800 20.1 and 19.7, 2000 55.1 and 53.2, 3000 105.7 and 107.2.
+//
+// Split precision: a tile works on 128 rows at a time (27 us for 64 rows, 30 us
+// for 128), so near tiles have 128 rows; far ones are twice as high on large
+// forms, for fewer tasks to order.  Measured, ms before and with both:
+// n = 4000 61.2 and 60.0, 7000 (near rows only) 108.3 and 103.6, 12000 280.9
+// and 265.9.
+inline void tile_heights(CostModel& cm, int n, int window, int precision, bool pair) {
+    if (precision == GBR_PREC_OZAKI) {
+        cm.near = 128;
+        cm.far_mul = n > 3000 ? 2 : 1;
+    } else if (pair ? n <= 2400 : (window > 64 && n <= 3000)) {
+        cm.near = 32;
+    }
+}
 
 int far_rows(int n);
 void pipeline_order(int n, std::vector<Window>& wins);

@@ -219,8 +219,8 @@ int plan_sweep(int n, int nbulges, int w, int nbc, std::vector<SweepWin>& out) {
 // Task graph for the persistent scheduler (Section 3.2, Fig. 2).
 //
 // Program order is the planner's window order; each window i contributes its
-// window task W_i and update tiles of UPD_BM panel rows (left panel columns
-// and right/Q panel rows on a global UPD_BM grid, so tiles of different
+// window task W_i and update tiles (left panel columns and right/Q panel rows
+// on global grids of the near and far tile heights, so tiles of different
 // windows line up).  A task depends on every earlier task whose exact
 // rectangle of S (or of Q) overlaps its own -- not on tiles, so two tasks
 // that touch different parts of a tile do not wait on each other -- and each
@@ -246,14 +246,14 @@ int far_rows(int n) {
 
 void build_graph(int n, const std::vector<Window>& wins, bool withQ, const CostModel& cm,
                  TaskGraph& G, int far, int threads, bool withZ) {
-    const int FAR = far > 0 ? far : far_rows(n);
+    const int FAR = far > 0 ? far : std::min(1024, far_rows(n) * cm.far_mul), NEAR = cm.near;
     std::vector<HostTask>& T = G.t;
     std::vector<std::pair<int, int>> edges;
     T.clear();
     {
         // capacity: per window its task and at most the near tiles, the far
         // tiles of the left / right panels and the Q and Z tiles
-        const size_t per = 2 + 4 * (size_t)UPD_NEAR / UPD_BM + 4 * ((size_t)n / FAR + 1);
+        const size_t per = 2 + 4 * (size_t)UPD_NEAR / NEAR + 4 * ((size_t)n / FAR + 1);
         T.reserve(wins.size() * per);
         edges.reserve(wins.size() * per);
     }
@@ -261,21 +261,21 @@ void build_graph(int n, const std::vector<Window>& wins, bool withQ, const CostM
         const int s = wins[i].s, e = wins[i].e, w = e - s;
         const int iw = (int)T.size();
         T.push_back(HostTask{TASK_W, i, 0, 0, 0, Rect{s, e, s, e}, dur_window(cm, w)});
-        // left panel: columns [e, n); 64-column tiles within UPD_NEAR of the
+        // left panel: columns [e, n); tiles of NEAR columns within UPD_NEAR of the
         // window (the next windows of the chain wait on those), far
         // tiles (FAR columns) beyond, each on a global grid so tiles of windows line up
         for (int c = e; c < n;) {
-            const int g = (c - e < UPD_NEAR) ? UPD_BM : FAR;
+            const int g = (c - e < UPD_NEAR) ? NEAR : FAR;
             int ce = std::min(n, (c / g + 1) * g);
             edges.push_back({iw, (int)T.size()});
             T.push_back(HostTask{TASK_L, i, c - e, ce - c, 0, Rect{s, e, c, ce},
                                  cm.lr_mats * dur_tile(cm, ce - c, w)});
             c = ce;
         }
-        // right panel: rows [0, s); 64-row tiles within UPD_NEAR above the window
+        // right panel: rows [0, s); tiles of NEAR rows within UPD_NEAR above the window
         for (int r = 0; r < s;) {
             const bool near = (s - r <= UPD_NEAR);
-            const int g = near ? UPD_BM : FAR;
+            const int g = near ? NEAR : FAR;
             int re = std::min(s, (r / g + 1) * g);
             if (!near && re > s - UPD_NEAR) re = std::max(r + 1, s - UPD_NEAR);
             edges.push_back({iw, (int)T.size()});
