@@ -83,7 +83,6 @@ METRIC = "selected eigenvalues reordered per second"
 NCU_TRAFFIC = {("n4000", "dmma"): 1.937360e9 + 2.652817e9,
                ("n4000", "fma"): 1.299070e9 + 2.728422e9,
                ("n4000", "ozaki"): 2.886808e9 + 4.348523e9,
-               ("eigvec4000", "evgemm"): 1.052943e9 + 0.125283e9,
                ("h4000", "persistent-dmma"): 0.220709e9 + 0.187885e9}
 
 
@@ -1269,24 +1268,21 @@ def run_eigvec(args, wl):
     if dist:
         dist.barrier()
     value, total_ms = whole_job_rate(n * args.steps, sum(ms), dist, "cuda")
-    pk, src = peaks()
-    fp64_peak = pk["bf16_tflops"] * (1.25 / 2250.0)
     ms_s = sum(s.ms_solve for s in sts) / len(sts)
     ms_b = sum(s.ms_backtransform for s in sts) / len(sts)
     f_s, f_b = sts[0].solve_flops, sts[0].backtransform_flops
     if ms_b >= ms_s:
-        roof = {"kernel": "evgemm_kernel (X = Q Y, DMMA)", "bound": "tensor",
+        roof = {"kernel": "evgemm_kernel (X = Q Y, FP64 FMA tiles)", "bound": "alu",
                 "achieved": f_b / (ms_b / 1e3) / 1e12, "unit": "TFLOP/s",
                 "flops_per_launch": f_b, "avg_launch_ms": ms_b,
                 "traffic": NCU_TRAFFIC.get((wl["name"], "evgemm"))}
     else:
-        roof = {"kernel": "eigvec_kernel (back substitution, FP64 FMA)", "bound": "alu",
+        roof = {"kernel": "evdiag_kernel, evupd_kernel (back substitution, FP64 FMA)", "bound": "alu",
                 "achieved": f_s / (ms_s / 1e3) / 1e12, "unit": "TFLOP/s",
                 "flops_per_launch": f_s, "avg_launch_ms": ms_s}
     roof.setdefault("traffic", None)
-    roof.update({"peak": fp64_peak, "frac": roof["achieved"] / fp64_peak,
-                 "peak_source": (f"{src} bf16 {pk['bf16_tflops']} TF/s x nominal FP64/bf16 "
-                                 "1.25/2250"),
+    roof.update({"peak": FP64_FMA_PEAK, "frac": roof["achieved"] / FP64_FMA_PEAK,
+                 "peak_source": FP64_FMA_PEAK_SOURCE,
                  "share_of_step": roof["avg_launch_ms"] / (total_ms / args.steps),
                  "other": {"solve_ms": ms_s, "solve_tflops": f_s / (ms_s / 1e3) / 1e12,
                            "backtransform_ms": ms_b,

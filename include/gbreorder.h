@@ -72,7 +72,7 @@ extern "C" {
 #define GBR_PREC_DMMA   0  /* off-diagonal updates on FP64 tensor cores (DMMA) */
 #define GBR_PREC_OZAKI  1  /* off-diagonal updates as split-precision emulated FP64:
                               7 signed 8-bit digit slices per operand, 28 exact
-                              bf16 tensor-core slice products, integer combination,
+                              fp16 tensor-core slice products, integer combination,
                               one rounding to double; the windows stay in FP64 */
 #define GBR_PREC_FMA    2  /* off-diagonal updates in FP64 on the FP64 FMA pipe (DFMA
                               register tiles, no tensor cores); same arithmetic
@@ -335,7 +335,7 @@ int gbr_reorder_noalloc(int n, double *S, int ldS, double *Q, int ldQ, const int
  *  8 precision  GBR_PREC_DMMA: FP64 tensor-core products (DMMA);
  *               GBR_PREC_FMA: FP64 fused multiply-adds, one chain per output
  *               over k in increasing order from +0 (register tiles);
- *               GBR_PREC_OZAKI: emulated FP64 on the bf16 tensor cores (7
+ *               GBR_PREC_OZAKI: emulated FP64 on the fp16 tensor cores (7
  *               balanced 8-bit digit slices of every entry, relative to
  *               the largest exponent of its row of Y or column of U; the 28
  *               slice products with p + q <= 8 summed exactly; one rounding
