@@ -1012,7 +1012,7 @@ def run_gen(args, wl):
         bf16_peak = pk["bf16_tflops"]
         work = 28.0 * st0.upd_flops + st0.win_flops * (bf16_peak / fp64_peak)
         achieved = work / (ms_k / 1e3) / 1e12
-        roof = {"kernel": "sched_kernel<pair> (persistent: pair window tasks + bf16 slice-product "
+        roof = {"kernel": "sched_kernel<pair> (persistent: pair window tasks + fp16 slice-product "
                           "tiles of S, T, Q, Z)",
                 "bound": "tensor", "achieved": achieved, "peak": bf16_peak, "unit": "TFLOP/s",
                 "frac": achieved / bf16_peak, "traffic": NCU_TRAFFIC.get((wl["name"], "ozaki")),
@@ -1385,7 +1385,7 @@ def measure_reorder(args, g, torch, dist, wl, prec, S_np, Q_np, sel, S, Q, S0, Q
     fp64_peak = pk["bf16_tflops"] * (1.25 / 2250.0)   # bf16 measured x nominal FP64/bf16
     cp_ms = sum(s.sched_cp_ms for s in stats) / len(stats)
     if ms_sched > 0 and prec == "ozaki":
-        # Split-precision updates: 28 bf16 slice products per FP64 product on
+        # Split-precision updates: 28 fp16 slice products per FP64 product on
         # the tensor pipe (the tiles run K = w densely); the window tasks stay
         # FP64.  frac counts the slice products only; frac_min_time adds the
         # time the FP64 window flops need at the FP64 peak.
@@ -1393,7 +1393,7 @@ def measure_reorder(args, g, torch, dist, wl, prec, S_np, Q_np, sel, S, Q, S0, Q
         slice_flops = 28.0 * flops_upd
         achieved = slice_flops / (ms_sched / 1e3) / 1e12
         min_s = slice_flops / (bf16_peak * 1e12) + flops_win / (fp64_peak * 1e12)
-        roof = {"kernel": "sched_kernel (persistent: FP64 window tasks + bf16 slice-product "
+        roof = {"kernel": "sched_kernel (persistent: FP64 window tasks + fp16 slice-product "
                           "update tiles)",
                 "bound": "tensor", "achieved": achieved, "peak": bf16_peak, "unit": "TFLOP/s",
                 "frac": achieved / bf16_peak,
