@@ -21,7 +21,9 @@ __device__ __forceinline__ double rsqrt_seed(double x) {
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     return y;
 }
-// x times 2^-1 for a normal x above the smallest binade.
+// x times 2^-1 for a normal x above the smallest binade, and for no other: the
+// exponent field of 0, of a subnormal or of an infinity gives a wrong number.
+// (In sqrt64 x is the seed of a normal number: within [2^-512, 2^511].)
 __device__ __forceinline__ double half_of(double x) {
     return __longlong_as_double(__double_as_longlong(x) - (1LL << 52));
 }

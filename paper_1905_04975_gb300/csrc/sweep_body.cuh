@@ -79,10 +79,12 @@ __device__ __forceinline__ void refl3(int len, double x0, double x1, double x2, 
     // reciprocal go into one correction: U's departure from orthogonality is 10
     // to 16% below that of tau = (b - x0) / b by CUDA's root and divisions, and
     // 1% above it without the correction, which takes 11 us of a window task.
+    // h is in [1/2, 1], so that it and y are normal and half_of holds; low, a
+    // rounding error, may be zero or below the normal range.
     const double p = fma(a2, a2, 1.0), q = fma(a1, a1, p);
     const double low = fma(a2, a2, 1.0 - p) + fma(a1, a1, p - q);
     const double h = half_of(q), y = rcp64(h);
-    *tau = fma(y, fma(-y, half_of(low), fma(-y, h, 1.0)), y);
+    *tau = fma(y, fma(-half_of(y), low, fma(-y, h, 1.0)), y);
     *beta = pos ? -nrm : nrm;
 }
 
