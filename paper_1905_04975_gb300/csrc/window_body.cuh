@@ -131,7 +131,8 @@ __device__ __forceinline__ bool sylv22_regs(const double* D, double* X) {
     unsigned long long ym = 0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) ym = abs_bits(y[c]) > ym ? abs_bits(y[c]) : ym;
-    if (!(ym < 0x7ff0000000000000ULL)) return false;  // inf or nan
+    // nan, or above 2^500: the full transform scales such a solution
+    if (!(ym < 0x5f30000000000000ULL)) return false;
     // un-permute: X[perm(c)] = y[c]   (X column-major 2x2, index i + 2k)
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
@@ -162,7 +163,10 @@ __device__ __forceinline__ bool sylv22_regs(const double* D, double* X) {
 // -sign(a0) |a| e_0: w0 = a0 + sign(a0) |a|, f = 2 / |w|^2 (taken from the
 // rounded w, so that only f's own rounding touches the orthogonality).  The
 // last component of w stays 1, so that applying it takes six FP64
-// instructions (a 3x3 product takes nine).
+// instructions (a 3x3 product takes nine).  The last component makes |w|^2 at
+// least 2, and a0, a1 are at most 2^500 (see sylv22_regs; a k = 3 solution
+// above 2^510 gives NaN or the identity, within the rounding errors of a
+// coupling that large): half_of holds.
 __device__ __forceinline__ void refl3(double a0, double a1, double* w0, double* f) {
     const double n1 = fma(a1, a1, 1.0);
     const double d = fabs(a0) + sqrt64(fma(a0, a0, n1));
@@ -199,10 +203,24 @@ static __device__ __noinline__ bool sylv22_full(const double* __restrict__ Sp, i
 // diagonal blocks shifted by B's first diagonal entry, which cancels) is
 // solved in closed form: M X = A C - C adj(B) with M = A^2 - tr(B) A + det(B) I
 // (Cayley-Hamilton on B), evaluated in FP32, then refined with FP64 residuals
-// until a correction c has |c| <= 2^-36 |X|: corrections shrink by the same
-// factor each time, and two of them that reach 2^-36 leave an error below
-// 2^-53.  Two corrections are the rule; a solution that does not get there in
-// six goes to the elimination with complete pivoting.
+// until, after at least two corrections, one is at most 2^-40 of the solution.
+// A correction can be small by luck while the next would not be, the more
+// easily the closer the blocks' eigenvalues; so a seeded solution has to leave
+// at most 2.5 eps max|D| in the block that must vanish, a quarter of what the
+// weak test allows.  One that does not, or has not converged in six
+// corrections, gives way to the elimination with complete pivoting under the
+// weak test itself.
+// Error in the block that must vanish, in eps max|D|, mean and largest of
+// 200 000 swaps of blocks with the same imaginary part and couplings of the
+// size of their separation s (host restatement, exact evaluation):
+//     s       elimination   2^-36, no limit   2^-40 and 2.5 eps
+//     1       0.49   2.8       0.42   2.8        0.42  2.4
+//     1e-2    0.39   2.5       0.39   2.6        0.39  2.4
+//     1e-4    0.39   2.5       0.40  12          0.39  2.5
+//     1e-5    0.39   2.5       0.40  94          0.39  2.5
+//     1e-6    0.39   2.9       0.66  1800        0.39  2.9
+// 2.00 corrections on average for s >= 0.1, 2.4 at 1e-2, 3.0 at 1e-3; below
+// 1e-5 most solutions are the elimination's.
 // FP64 instructions: 3 + 5 per correction, 30 for the reflectors, 22 for the
 // products and tests; the elimination in FP64, two square roots and five
 // divisions took about 200.
@@ -229,6 +247,8 @@ __device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, i
     t1 = __shfl_xor_sync(hmask, mx, 8);
     mx = t1 > mx ? t1 : mx;
     const unsigned long long tb = thresh_bits(mx);
+    // a quarter of it for a seeded solution (exponent arithmetic)
+    const unsigned long long tb4 = tb > (3ULL << 52) ? tb - (2ULL << 52) : tb;
     // FP32 copies, scaled by the power of two of the largest entry of A and B
     int em = 0;
     {
@@ -286,71 +306,76 @@ __device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, i
         const float dmax = spread(to_f32(res, eoff));
         own += from_f32(k ? (i ? x[3] : x[2]) : (i ? x[1] : x[0]));
         if (!(dmax <= 0.25f * xmax)) break;  // also NaN: no convergence
-        if (it > 0 && dmax <= 1.4551915e-11f * xmax) { good = xmax < 1e30f; break; }
+        if (it > 0 && dmax <= 9.094947e-13f * xmax) { good = xmax < 1e30f; break; }  // 2^-40
     }
 #pragma unroll
     for (int t = 0; t < 4; ++t) X[t] = __shfl_sync(hmask, own, hbase + t);
-    if (!good) {
-        double Xf[4];
-        if (!sylv22_full(Sp, ja, Xf)) return false;
+#pragma unroll 1
+    for (;; good = false) {
+        if (!good) {
+            double Xf[4];
+            if (!sylv22_full(Sp, ja, Xf)) return false;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) X[t] = Xf[t];
-    }
-    // reflector 1 on column 0 of [-X; I], (-x00, -x10, 1, 0); reflector 2 on
-    // rows 1..3 of reflector 1 times column 1, (-x01, -x11, 0, 1)
-    const double w1 = -X[1];
-    double w0, f1, u0, f2;
-    refl3(-X[0], w1, &w0, &f1);
-    const double s1 = fma(w0, -X[2], w1 * -X[3]) * f1;
-    const double q1 = fma(-s1, w1, -X[3]), u1 = -s1;  // (q1, u1, 1)
-    refl3(q1, u1, &u0, &f2);
-    // Qs = (I - f1 w w^T)(I - f2 u u^T), w = (w0, w1, 1, 0), u = (0, u0, u1, 1)
-    const double wu = fma(w1, u0, u1);
-    const double wr = sel4(r, w0, w1, 1.0, 0.0), wc = sel4(c, w0, w1, 1.0, 0.0);
-    const double ur = sel4(r, 0.0, u0, u1, 1.0), uc = sel4(c, 0.0, u0, u1, 1.0);
-    const double ar = f1 * wr;
-    double qs = fma(-ar, wc, (r == c) ? 1.0 : 0.0);
-    qs = fma(-(f2 * uc), fma(-ar, wu, ur), qs);
-    // T = Qs^T D: T[r][c] = sum_a Qs[a][r] D[a][c]
-    double T = __shfl_sync(hmask, qs, hbase + 0 + 4 * r) * dc0;
-    T = fma(__shfl_sync(hmask, qs, hbase + 1 + 4 * r), dc1, T);
-    T = fma(__shfl_sync(hmask, qs, hbase + 2 + 4 * r), dc2, T);
-    T = fma(__shfl_sync(hmask, qs, hbase + 3 + 4 * r), dc3, T);
-    // Dt = T Qs: Dt[r][c] = sum_b T[r][b] Qs[b][c]
-    double Dt = 0.0;
-#pragma unroll
-    for (int bb = 0; bb < 4; ++bb)
-        Dt = fma(__shfl_sync(hmask, T, hbase + r + 4 * bb), __shfl_sync(hmask, qs, hbase + bb + 4 * c),
-                 Dt);
-    // weak test on the lower-left 2x2 block
-    const bool low = (r >= 2 && c < 2);
-    const bool weak_bad = low && abs_bits(Dt) > tb;
-    if (__any_sync(hmask, weak_bad)) return false;
-    const double Dt0 = low ? 0.0 : Dt;
-    if (strong) {
-        // P = Qs Dt0: P[r][b] = sum_a Qs[r][a] Dt0[a][b]
-        double P = 0.0;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-            P = fma(__shfl_sync(hmask, qs, hbase + r + 4 * a), __shfl_sync(hmask, Dt0, hbase + a + 4 * c),
-                    P);
-        // E = P Qs^T - D: E[r][c] = sum_b P[r][b] Qs[c][b] - D[r][c]
-        double E = 0.0;
+            for (int t = 0; t < 4; ++t) X[t] = Xf[t];
+        }
+        // reflector 1 on column 0 of [-X; I], (-x00, -x10, 1, 0); reflector 2 on
+        // rows 1..3 of reflector 1 times column 1, (-x01, -x11, 0, 1)
+        const double w1 = -X[1];
+        double w0, f1, u0, f2;
+        refl3(-X[0], w1, &w0, &f1);
+        const double s1 = fma(w0, -X[2], w1 * -X[3]) * f1;
+        const double q1 = fma(-s1, w1, -X[3]), u1 = -s1;  // (q1, u1, 1)
+        refl3(q1, u1, &u0, &f2);
+        // Qs = (I - f1 w w^T)(I - f2 u u^T), w = (w0, w1, 1, 0), u = (0, u0, u1, 1)
+        const double wu = fma(w1, u0, u1);
+        const double wr = sel4(r, w0, w1, 1.0, 0.0), wc = sel4(c, w0, w1, 1.0, 0.0);
+        const double ur = sel4(r, 0.0, u0, u1, 1.0), uc = sel4(c, 0.0, u0, u1, 1.0);
+        const double ar = f1 * wr;
+        double qs = fma(-ar, wc, (r == c) ? 1.0 : 0.0);
+        qs = fma(-(f2 * uc), fma(-ar, wu, ur), qs);
+        // T = Qs^T D: T[r][c] = sum_a Qs[a][r] D[a][c]
+        double T = __shfl_sync(hmask, qs, hbase + 0 + 4 * r) * dc0;
+        T = fma(__shfl_sync(hmask, qs, hbase + 1 + 4 * r), dc1, T);
+        T = fma(__shfl_sync(hmask, qs, hbase + 2 + 4 * r), dc2, T);
+        T = fma(__shfl_sync(hmask, qs, hbase + 3 + 4 * r), dc3, T);
+        // Dt = T Qs: Dt[r][c] = sum_b T[r][b] Qs[b][c]
+        double Dt = 0.0;
 #pragma unroll
         for (int bb = 0; bb < 4; ++bb)
-            E = fma(__shfl_sync(hmask, P, hbase + r + 4 * bb), __shfl_sync(hmask, qs, hbase + c + 4 * bb),
-                    E);
-        E -= sel4(r, dc0, dc1, dc2, dc3);
-        if (__any_sync(hmask, abs_bits(E) > tb)) return false;
+            Dt = fma(__shfl_sync(hmask, T, hbase + r + 4 * bb),
+                     __shfl_sync(hmask, qs, hbase + bb + 4 * c), Dt);
+        // weak test on the lower-left 2x2 block
+        const bool low = (r >= 2 && c < 2);
+        bool pass = !__any_sync(hmask, low && abs_bits(Dt) > (good ? tb4 : tb));
+        const double Dt0 = low ? 0.0 : Dt;
+        if (strong && pass) {
+            // P = Qs Dt0: P[r][b] = sum_a Qs[r][a] Dt0[a][b]
+            double P = 0.0;
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+                P = fma(__shfl_sync(hmask, qs, hbase + r + 4 * a),
+                        __shfl_sync(hmask, Dt0, hbase + a + 4 * c), P);
+            // E = P Qs^T - D: E[r][c] = sum_b P[r][b] Qs[c][b] - D[r][c]
+            double E = 0.0;
+#pragma unroll
+            for (int bb = 0; bb < 4; ++bb)
+                E = fma(__shfl_sync(hmask, P, hbase + r + 4 * bb),
+                        __shfl_sync(hmask, qs, hbase + c + 4 * bb), E);
+            E -= sel4(r, dc0, dc1, dc2, dc3);
+            pass = !__any_sync(hmask, abs_bits(E) > tb);
+        }
+        if (pass) {
+            z[0] = w0;
+            z[1] = w1;
+            z[2] = f1;
+            z[3] = u0;
+            z[4] = u1;
+            z[5] = f2;
+            *dnrc = Dt0;
+            return true;
+        }
+        if (!good) return false;
     }
-    z[0] = w0;
-    z[1] = w1;
-    z[2] = f1;
-    z[3] = u0;
-    z[4] = u1;
-    z[5] = f2;
-    *dnrc = Dt0;
-    return true;
 }
 
 // k = 3 swap by four lanes (all 32 lanes of the warp call it, eight swaps at a
