@@ -89,6 +89,11 @@ __device__ __forceinline__ double pick8(const double (&v)[8], int i) {
     return r;
 }
 
+// An eighth of a threshold (a bit pattern, exponent arithmetic).
+__device__ __forceinline__ unsigned long long thresh_eighth(unsigned long long t) {
+    return t > (4ULL << 52) ? t - (3ULL << 52) : t;
+}
+
 // The elimination with complete pivoting in FP64, for the swaps whose
 // FP32-seeded solution does not converge (out of line: it is rare).  Returns
 // unknown l on lane l < N; *g is its scaling against overflow.
@@ -211,17 +216,17 @@ static __device__ __noinline__ double gen_sylv_full(int p, int q, const double* 
 
 // The same system solved by an FP32 inverse (Gauss-Jordan in place, rows on
 // lanes, partial pivoting without exchanging rows) and refined with FP64
-// residuals until a correction is at most 2^-36 of the solution (the
-// correction after it would be below 2^-53, see swap22_halfwarp in
-// window_body.cuh).  The equations of A and of B are scaled by the power of
+// residuals until, after at least two corrections, one is at most 2^-40 of the
+// solution, at most six times.  The equations of A and of B are scaled by the power of
 // two of the matrix's largest entry; ea, eb: those exponent fields.  Returns
-// unknown l on lane l < N, *good on all lanes.
+// unknown l on lane l < N; *level on all lanes: 2 if the last correction was at
+// most 2^-40 of the solution, 1 if at most 2^-36, else 0.
 //
 // Five FP64 instructions a correction, two corrections as a rule; the
 // elimination in FP64 takes about 20 per unknown and a dependent division.
 __device__ __forceinline__ double gen_sylv_seeded(int p, int q, const double* __restrict__ DA,
                                                   const double* __restrict__ DB, int l, int ob,
-                                                  unsigned om, int ea, int eb, bool* good) {
+                                                  unsigned om, int ea, int eb, int* level) {
     const int sp = p - 1, pq = p * q, N = 2 * pq;  // division by p is a shift
     // row l: X11[i][:] R[:][cc] - L[i][:] X22[:][cc] = -X12[i][cc], X = A or B
     const int eq = l >= pq, rem = l - (eq ? pq : 0), i = rem & sp, cc = rem >> sp;
@@ -289,7 +294,7 @@ __device__ __forceinline__ double gen_sylv_seeded(int p, int q, const double* __
     const float xmax = omax(x);
     double y = from_f32(x);
     const int r0 = ob + (row ? cc << sp : 0), l0 = ob + (row ? pq + i : 0);
-    *good = false;
+    float dmax = __int_as_float(0x7f800000);
 #pragma unroll 1
     for (int it = 0; it < 6 && !singular; ++it) {
         double res = fma(-c0, __shfl_sync(om, y, r0), b);
@@ -297,17 +302,22 @@ __device__ __forceinline__ double gen_sylv_seeded(int p, int q, const double* __
         res = fma(-c1, __shfl_sync(om, y, r0 + sp), res);
         res = fma(d1, __shfl_sync(om, y, q == 2 ? l0 + p : l0), res);
         x = solve(to_f32(res, eoff));
-        const float dmax = omax(x);
+        dmax = omax(x);
         y += from_f32(x);
         if (!(dmax <= 0.25f * xmax)) break;  // also NaN: no convergence
-        if (it > 0 && dmax <= 1.4551915e-11f * xmax) { *good = xmax < 1e30f; break; }
+        if (it > 0 && dmax <= 9.094947e-13f * xmax) break;
     }
+    *level = !(xmax < 1e30f && dmax <= 1.4551915e-11f * xmax) ? 0 : (dmax <= 9.094947e-13f * xmax ? 2 : 1);
     return y;
 }
 
 // Reflector I - f w w^T on 4-vectors mapping (a0, a1, a2, a3) onto
 // -sign(a0) |a| e_0: w = (w0, a1, a2, a3), f = 2 / |w|^2 from the rounded w.
-// |a| is in the normal range: one of a1..a3 is 1 (or the solution's scaling).
+// One of a1..a3 is 1, so that |w|^2 is at least 2 and half_of holds; or it is
+// the solution's scaling g < 1, and then another entry of the solution is next
+// to overflow: its own reflector is NaN and the swap fails its tests.  (The
+// same for entries above 2^511; between 2^510 and that f is 0 and the factor
+// the identity, and the tests decide.)
 __device__ __forceinline__ void refl4(double a0, double a1, double a2, double a3, double* w0,
                                       double* f) {
     const double sg = fma(a1, a1, fma(a2, a2, a3 * a3));
@@ -381,111 +391,132 @@ __device__ __forceinline__ bool gen_swap_octet(int p, int q, const double* __res
     }
 
     // --- generalized Sylvester equation: unknowns [vec R; vec L] on lanes
-    double g = 1.0;
-    bool good;
-    double y = gen_sylv_seeded(p, q, DA, DB, l, ob, om, ea, eb, &good);
-    if (!good) y = gen_sylv_full(p, q, DA, DB, l, ob, om, &g);
-    // --- QR factor: column (l & 3) of Qs (lanes 0-3, from [L; g I]) or of
-    // Zs (lanes 4-7, from [R; g I]); H1 for column 0, H2 on rows 1..3
-    {
-        double X[4];
+    // A seeded solution's corrections can be small by luck while the next one
+    // would not be, the more easily the closer the eigenvalues: it has to leave
+    // at most 2.5 eps ||.||_F in the blocks that must vanish, an eighth of what
+    // the weak test allows.  Otherwise the elimination takes its place; and
+    // where that fails the tests (its pivots do not see the scales of the two
+    // equations), a seeded solution that comes to 2^-36.  Largest error in eps
+    // and swaps rejected, 160 000 swaps each, couplings of the size of the
+    // separation (host restatement, exact evaluation):
+    //                     elimination    2^-36, no limit   this rule
+    //   1|1, apart 1e-4     2.2    0         25    3        2.0    0
+    //   1|1, apart 1e-6     2.0    0       3500  577        2.4    0
+    //   2|2, apart 1e-4     2.3    0        4.6    0        1.7    0
+    //   2|2, apart 1e-6     2.2    0       1800  200        2.2    0
+    int level;
+    const double ys = gen_sylv_seeded(p, q, DA, DB, l, ob, om, ea, eb, &level);
+#pragma unroll 1
+    for (int att = level == 2 ? 0 : 1;; ++att) {
+        double g = 1.0, y = ys;
+        if (att == 1) y = gen_sylv_full(p, q, DA, DB, l, ob, om, &g);
+        const unsigned long long lima = att == 0 ? thresh_eighth(tha) : tha;
+        const unsigned long long limb = att == 0 ? thresh_eighth(thb) : thb;
+        // --- QR factor: column (l & 3) of Qs (lanes 0-3, from [L; g I]) or of
+        // Zs (lanes 4-7, from [R; g I]); H1 for column 0, H2 on rows 1..3
+        {
+            double X[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const double v = __shfl_sync(om, y, ob + (t < pq ? (zhalf ? t : pq + t) : 0));
-            X[t] = t < pq ? v : 0.0;
-        }
-        // [X; g I]: columns (X0, X1, g, 0), (X2, X3, 0, g) for p = 2,
-        // (X0, g, 0, 0), (X1, 0, g, 0) for p = 1
-        const double a1 = p == 2 ? X[1] : g, a2 = p == 2 ? g : 0.0;
-        double w0, f1;
-        refl4(X[0], a1, a2, 0.0, &w0, &f1);
-        double u0 = 1.0, u1 = 0.0, u2 = 0.0, f2 = 0.0;
-        if (q == 2) {
-            const double m0 = p == 2 ? X[2] : X[1], m1 = p == 2 ? X[3] : 0.0, m2 = p == 2 ? 0.0 : g;
-            const double d = fma(w0, m0, fma(a1, m1, a2 * m2)) * f1;
-            const double x1 = fma(-d, a1, m1);
-            u1 = fma(-d, a2, m2);
-            u2 = p == 2 ? g : 0.0;
-            refl4(x1, u1, u2, 0.0, &u0, &f2);
-        }
-        // column c of H1 diag(1, H2): z = diag(1, H2) e_c, then H1 z
-        const int c = l & 3;
-        const double uc = f2 * (c == 1 ? u0 : (c == 2 ? u1 : (c == 3 ? u2 : 0.0)));
-        const double z0 = c == 0 ? 1.0 : 0.0, z1 = fma(-uc, u0, c == 1 ? 1.0 : 0.0);
-        const double z2 = fma(-uc, u1, c == 2 ? 1.0 : 0.0), z3 = fma(-uc, u2, c == 3 ? 1.0 : 0.0);
-        const double d = fma(w0, z0, fma(a1, z1, a2 * z2)) * f1;
-        double* out = sc + (zhalf ? SC_Z : SC_Q) + c * 4;
-        out[0] = fma(-d, w0, z0);
-        out[1] = fma(-d, a1, z1);
-        out[2] = fma(-d, a2, z2);
-        out[3] = z3;
-    }
-    __syncwarp(om);
-    const double* Qs = sc + SC_Q;
-    const double* Zs = sc + SC_Z;
-    // --- W = Qs^T D (own entries), then N = W Zs
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        const int r = er + t;
-        double wa = 0.0, wb = 0.0;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            wa = fma(Qs[r * 4 + a], DA[ec * 4 + a], wa);
-            wb = fma(Qs[r * 4 + a], DB[ec * 4 + a], wb);
-        }
-        sc[SC_WA + ec * 4 + r] = wa;
-        sc[SC_WB + ec * 4 + r] = wb;
-    }
-    __syncwarp(om);
-    bool low = false;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        const int r = er + t;
-        double na = 0.0, nb = 0.0;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            na = fma(sc[SC_WA + a * 4 + r], Zs[ec * 4 + a], na);
-            nb = fma(sc[SC_WB + a * 4 + r], Zs[ec * 4 + a], nb);
-        }
-        // weak test on the block that must vanish: rows [q, k) x columns [0, q)
-        if (ec < q && r >= q && r < k) {
-            low |= mag(na) > tha || mag(nb) > thb;
-            na = 0.0;
-            nb = 0.0;
-        }
-        sc[SC_NA + ec * 4 + r] = na;
-        sc[SC_NB + ec * 4 + r] = nb;
-    }
-    if (__any_sync(om, low)) return false;
-    __syncwarp(om);
-    if (strong) {
-        // V = Qs N (into W), then D - V Zs^T must stay below the thresholds
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const int r = er + t;
-            double va = 0.0, vb = 0.0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                va = fma(Qs[a * 4 + r], sc[SC_NA + ec * 4 + a], va);
-                vb = fma(Qs[a * 4 + r], sc[SC_NB + ec * 4 + a], vb);
+            for (int t = 0; t < 4; ++t) {
+                const double v = __shfl_sync(om, y, ob + (t < pq ? (zhalf ? t : pq + t) : 0));
+                X[t] = t < pq ? v : 0.0;
             }
-            sc[SC_WA + ec * 4 + r] = va;
-            sc[SC_WB + ec * 4 + r] = vb;
+            // [X; g I]: columns (X0, X1, g, 0), (X2, X3, 0, g) for p = 2,
+            // (X0, g, 0, 0), (X1, 0, g, 0) for p = 1
+            const double a1 = p == 2 ? X[1] : g, a2 = p == 2 ? g : 0.0;
+            double w0, f1;
+            refl4(X[0], a1, a2, 0.0, &w0, &f1);
+            double u0 = 1.0, u1 = 0.0, u2 = 0.0, f2 = 0.0;
+            if (q == 2) {
+                const double m0 = p == 2 ? X[2] : X[1], m1 = p == 2 ? X[3] : 0.0, m2 = p == 2 ? 0.0 : g;
+                const double d = fma(w0, m0, fma(a1, m1, a2 * m2)) * f1;
+                const double x1 = fma(-d, a1, m1);
+                u1 = fma(-d, a2, m2);
+                u2 = p == 2 ? g : 0.0;
+                refl4(x1, u1, u2, 0.0, &u0, &f2);
+            }
+            // column c of H1 diag(1, H2): z = diag(1, H2) e_c, then H1 z
+            const int c = l & 3;
+            const double uc = f2 * (c == 1 ? u0 : (c == 2 ? u1 : (c == 3 ? u2 : 0.0)));
+            const double z0 = c == 0 ? 1.0 : 0.0, z1 = fma(-uc, u0, c == 1 ? 1.0 : 0.0);
+            const double z2 = fma(-uc, u1, c == 2 ? 1.0 : 0.0), z3 = fma(-uc, u2, c == 3 ? 1.0 : 0.0);
+            const double d = fma(w0, z0, fma(a1, z1, a2 * z2)) * f1;
+            double* out = sc + (zhalf ? SC_Z : SC_Q) + c * 4;
+            out[0] = fma(-d, w0, z0);
+            out[1] = fma(-d, a1, z1);
+            out[2] = fma(-d, a2, z2);
+            out[3] = z3;
         }
         __syncwarp(om);
-        bool bad = false;
+        const double* Qs = sc + SC_Q;
+        const double* Zs = sc + SC_Z;
+        // --- W = Qs^T D (own entries), then N = W Zs
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             const int r = er + t;
-            double va = 0.0, vb = 0.0;
+            double wa = 0.0, wb = 0.0;
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                va = fma(sc[SC_WA + a * 4 + r], Zs[a * 4 + ec], va);
-                vb = fma(sc[SC_WB + a * 4 + r], Zs[a * 4 + ec], vb);
+                wa = fma(Qs[r * 4 + a], DA[ec * 4 + a], wa);
+                wb = fma(Qs[r * 4 + a], DB[ec * 4 + a], wb);
             }
-            bad |= mag(va - DA[ec * 4 + r]) > tha || mag(vb - DB[ec * 4 + r]) > thb;
+            sc[SC_WA + ec * 4 + r] = wa;
+            sc[SC_WB + ec * 4 + r] = wb;
         }
-        if (__any_sync(om, bad)) return false;
+        __syncwarp(om);
+        bool low = false;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int r = er + t;
+            double na = 0.0, nb = 0.0;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                na = fma(sc[SC_WA + a * 4 + r], Zs[ec * 4 + a], na);
+                nb = fma(sc[SC_WB + a * 4 + r], Zs[ec * 4 + a], nb);
+            }
+            // weak test on the block that must vanish: rows [q, k) x columns [0, q)
+            if (ec < q && r >= q && r < k) {
+                low |= mag(na) > lima || mag(nb) > limb;
+                na = 0.0;
+                nb = 0.0;
+            }
+            sc[SC_NA + ec * 4 + r] = na;
+            sc[SC_NB + ec * 4 + r] = nb;
+        }
+        bool fail = __any_sync(om, low);
+        __syncwarp(om);
+        if (strong && !fail) {
+            // V = Qs N (into W), then D - V Zs^T must stay below the thresholds
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const int r = er + t;
+                double va = 0.0, vb = 0.0;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    va = fma(Qs[a * 4 + r], sc[SC_NA + ec * 4 + a], va);
+                    vb = fma(Qs[a * 4 + r], sc[SC_NB + ec * 4 + a], vb);
+                }
+                sc[SC_WA + ec * 4 + r] = va;
+                sc[SC_WB + ec * 4 + r] = vb;
+            }
+            __syncwarp(om);
+            bool bad = false;
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const int r = er + t;
+                double va = 0.0, vb = 0.0;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    va = fma(sc[SC_WA + a * 4 + r], Zs[a * 4 + ec], va);
+                    vb = fma(sc[SC_WB + a * 4 + r], Zs[a * 4 + ec], vb);
+                }
+                bad |= mag(va - DA[ec * 4 + r]) > tha || mag(vb - DB[ec * 4 + r]) > thb;
+            }
+            fail = __any_sync(om, bad);
+        }
+        if (!fail) break;
+        if (att == 2 || (att == 1 && level == 0)) return false;
+        __syncwarp(om);
     }
     // --- T stays upper triangular: rotate the two columns of each new 2x2
     // block (lanes 0-3: rows of NA, lanes 4-7: rows of NB, then all of Zs).

@@ -1,11 +1,11 @@
 """Single swaps of close eigenvalues are as exact as those of separated ones.
 
-A form of decoupled quads: 64 or 32 pairs of neighbouring blocks, coupled only
+A form of decoupled quads: 16 to 64 pairs of neighbouring blocks, coupled only
 within the pair, the lower block of each selected.  Its window's first step
 swaps every pair; the exchanges between pairs that follow have a zero coupling,
 so that their Sylvester solutions are zero and their transformations exact
 permutations.  Q then holds each pair's own transformation, and the part of
-Q^T D Q that the swap has to make vanish is evaluated in extended
+Q^T D Q (Q^T D Z) that the swap has to make vanish is evaluated in extended
 precision.
 
 Against the same statistic at a separation of 1: only the Sylvester solution
@@ -102,5 +102,42 @@ def test_window_swaps(gbr, size):
     ref = window_errors(gbr, 1.0, 1, size)
     for i, sep in enumerate([1e-2, 1e-3, 1e-4, 3e-5, 1e-5, 3e-6, 1e-6, 1e-7]):
         e = window_errors(gbr, sep, 10 + i, size)
+        assert e.max() <= 2.0 * ref.max(), sep
+        assert e.mean() <= 1.25 * ref.mean(), sep
+
+
+def gen_errors(g, sep, seed, size, count=60):
+    """The same for pairs (S, T), with T's diagonal in [1, 2]; every swap has
+    to be accepted, as a backward stable one is."""
+    pairs = 64 // (2 * size)
+    rng = np.random.default_rng(seed)
+    M = quads(rng, count, pairs, size, sep)
+    k = 2 * size
+    B = sep * np.triu(rng.standard_normal((count, pairs, k, k)), 1)
+    for i in range(k):
+        B[..., i, i] = rng.uniform(1.0, 2.0, (count, pairs))
+    A = np.zeros_like(M)
+    for o in (0, size):  # diagonal blocks T_b M_b, so that S T^-1 has M's eigenvalues
+        A[..., o:o + size, o:o + size] = B[..., o:o + size, o:o + size] @ M[..., o:o + size, o:o + size]
+    A[..., :size, size:] = M[..., :size, size:]
+    S, T = assemble(A), assemble(B)
+    n = S.shape[1]
+    sel = np.tile(np.repeat([0, 1], size), pairs).astype(np.int32)
+    Qs, Zs, rejected = [], [], 0
+    for s, t in zip(S, T):
+        d = [g.to_device(x) for x in (s, t, np.eye(n), np.eye(n))]
+        rejected += g.reorder_gen(*d, sel, window=64, chain=32).status
+        Qs.append(g.to_host(d[2]))
+        Zs.append(g.to_host(d[3]))
+    assert rejected == 0, (sep, rejected)
+    Q, Z = pair_factors(np.array(Qs), pairs, size), pair_factors(np.array(Zs), pairs, size)
+    return np.maximum(vanishing(A, Q, Z, size), vanishing(B, Q, Z, size))
+
+
+@pytest.mark.parametrize("size", [1, 2])
+def test_pair_swaps(gbr, size):
+    ref = gen_errors(gbr, 1.0, 1, size, 120)
+    for i, sep in enumerate([1e-2, 1e-3, 1e-4, 3e-5, 1e-5, 3e-6, 1e-6, 1e-7]):
+        e = gen_errors(gbr, sep, 10 + i, size, 120)
         assert e.max() <= 2.0 * ref.max(), sep
         assert e.mean() <= 1.25 * ref.mean(), sep
