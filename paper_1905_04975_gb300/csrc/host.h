@@ -8,6 +8,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <functional>
 #include <memory>
 #include <mutex>
@@ -137,12 +138,21 @@ struct CostModel {
 // server, which fill the device with many problems, keep the defaults.
 //
 // FP64: the next window of a chain waits for a near tile of 64 rows (210 us at
-// w = 128, beside a window task of 1.3 ms).  On a small form most SMs wait
-// anyway, and tiles of 32 rows halve that; on a large one the device is full
-// and the second load of U per 64 rows costs.  Measured, ms with 64 and 32
-// rows, w = 128: n = 600 8.83 and 8.26, 1200 18.8 and 17.6, 2200 36.3 and 35.7,
-// 3000 57.0 and 56.6, 4000 96.3 and 99.0; w = 64: n = 1500 15.7 and 16.1; pairs
-// (w = 64): n = 800 20.1 and 19.7, 2000 55.1 and 53.2, 3000 105.7 and 107.2.
+// w = 128, beside a window task of 1.3 ms).  On a small form of wide windows
+// most SMs wait anyway, and tiles of 32 rows halve that; with n / w windows in
+// a chain's range the device fills up, there are twice as many near tiles to
+// claim, and each loads U.  The tensor-core tile (DMMA) loads its operands per
+// 64 rows and gains less.  Measured, ms with 64 and 32 rows:
+//   FMA   w = 128: n = 600 9.35 and 8.82, 1500 24.9 and 23.1, 2500 42.0 and
+//         41.3, 3000 56.7 and 56.4; w = 96: 600 7.42 and 6.97, 2500 35.3 and
+//         34.9, 3000 52.2 and 52.4; w = 72: 600 5.95 and 5.71, 1500 17.9 and
+//         17.9, 2500 37.5 and 38.4, 3000 55.0 and 58.1
+//   DMMA  w = 128: n = 1500 27.5 and 26.6, 2500 46.8 and 47.5; w = 96: 1500
+//         23.2 and 23.4, 3000 60.6 and 64.6; w = 72: 3000 60.3 and 68.3
+//   pairs, FMA   w = 64: n = 800 20.0 and 19.4, 2000 54.5 and 52.2, 2100 58.8
+//         and 57.3, 2400 72.5 and 73.6; w = 32: 800 19.9 and 21.1, 2400 95.5
+//         and 112.8; w = 16: 2400 292 and 350
+//   pairs, DMMA  w = 64: n = 2000 58.4 and 60.1; w = 32: 2400 138 and 160
 //
 // Split precision: a tile works on 128 rows at a time (27 us for 64 rows, 30 us
 // for 128), so near tiles have 128 rows; far ones are twice as high on large
@@ -153,8 +163,11 @@ inline void tile_heights(CostModel& cm, int n, int window, int precision, bool p
     if (precision == GBR_PREC_OZAKI) {
         cm.near = 128;
         cm.far_mul = n > 3000 ? 2 : 1;
-    } else if (pair ? n <= 2400 : (window > 64 && n <= 3000)) {
-        cm.near = 32;
+    } else {
+        const bool fma = precision == GBR_PREC_FMA;
+        if (pair ? fma && window > 48 && n <= 34 * window
+                 : (fma ? window > 64 && n <= std::min(27 * window, 3000) : window > 96 && n <= 16 * window))
+            cm.near = 32;
     }
 }
 
