@@ -1372,10 +1372,11 @@ def measure_reorder(args, g, torch, dist, wl, prec, S_np, Q_np, sel, S, Q, S0, Q
     # kernel runs every window task and update tile; a large pass runs as
     # three consecutive launches of it (the host orders the later chunks'
     # task graphs while the earlier ones run).  The other launches of a step
-    # are the validation, block-scan and eigenvalue kernels (no swap of these
-    # workloads is rejected, so there is no re-planning scan).
+    # are the validation (which also reads the block pattern) and eigenvalue
+    # kernels (no swap of these workloads is rejected, so there is no
+    # re-planning scan).
     st0 = stats[0]
-    nsched = max(1, int(st0.launches) - 3)
+    nsched = max(1, int(st0.launches) - 2)
     nwin = st0.windows
     flops_upd = st0.upd_flops
     flops_win = st0.win_flops
