@@ -402,7 +402,10 @@ static int reorder_device_at(char* b, char* stage, int n, double* S, int ldS, do
     // after a pass: eigenvalues (those of the result if nothing was rejected)
     // and counters, in one copy that the pass's own wait covers
     auto fetch = [&]() -> int {
-        if (want_eig) GBR_CK(launch_eigs(n, S, ldS, d_eig, d_eig + n, st), "eigenvalue kernel");
+        if (want_eig) {
+            GBR_CK(launch_eigs(n, S, ldS, d_eig, d_eig + n, st), "eigenvalue kernel");
+            launches += 1;
+        }
         const size_t bytes = want_eig ? off_eig + 2 * sizeof(double) * (size_t)n : sizeof(DevCounters);
         GBR_CK(cudaMemcpyAsync(stage, b, bytes, cudaMemcpyDeviceToHost, st), "D2H counters");
         return 0;
@@ -467,7 +470,6 @@ static int reorder_device_at(char* b, char* stage, int n, double* S, int ldS, do
     }
     if (eig_re) memcpy(eig_re, h_eig, n * sizeof(double));
     if (eig_im) memcpy(eig_im, h_eig + n, n * sizeof(double));
-    if (want_eig) launches += 1;
     double msw = 0.0, msu = 0.0;
     for (size_t i = 0; i + 1 < evw.size(); i += 2) {
         float t = 0.f;
