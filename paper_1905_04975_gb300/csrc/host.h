@@ -204,7 +204,7 @@ struct SchedLaunch {
     int* ctl = nullptr;               // head, err (and spare words), 256 bytes
     size_t trace_bytes = 0;
     std::vector<SchedTask> tq;        // host copy of the queue (trace decoding)
-    std::unique_ptr<char[]> image;    // host source of the upload (kept until it has run)
+    std::unique_ptr<char[]> image;    // host source of an upload that is not waited for
 };
 
 // Plans the task graph of all instances, orders it for `grid` CTAs, and

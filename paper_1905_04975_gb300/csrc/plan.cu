@@ -714,6 +714,7 @@ int sched_prepare(std::vector<InstPlan>& plans, const gbr_opts& o, const CostMod
     L->trace_bytes = b_tr;
     L->tq.clear();
     if (b_tr) L->tq.assign(tq, tq + nt);
+    if (wait) L->image.reset();  // a planned batch lives on
     return 0;
 }
 
