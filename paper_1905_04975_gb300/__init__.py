@@ -292,7 +292,7 @@ def update_panel(Y, U, precision="dmma", *, stream=None) -> None:
     Y: 2-D float64 CUDA tensor (rows x w) with stride 1 along one dimension
     (row- or column-major); U: w x w column-major float64 CUDA tensor.
     precision: "dmma" (FP64 tensor cores) or "ozaki" (emulated FP64 on the
-    bf16 tensor cores)."""
+    fp16 tensor cores)."""
     lib = load()
     rows, w = int(Y.shape[0]), int(Y.shape[1])
     if str(Y.dtype) != "torch.float64" or str(U.dtype) != "torch.float64":

@@ -20,8 +20,6 @@
 #include "common.cuh"
 #include "window_body.cuh"
 
-#include <cuda_bf16.h>
-
 namespace gbr {
 namespace upd {
 

@@ -156,8 +156,9 @@ __device__ __forceinline__ bool sylv22_regs(const double* D, double* X) {
 // task of w = 128, m = 64 took 1.90 ms and takes 1.48 ms (median in the
 // n = 4000 schedule), one of w = 32, m = 16 took 268 us and took 193 us (1.31
 // ms and 145 us since the control of a step runs beside the critical products
-// and a lane of a product warp works on two items at once); the rounding errors of whole reorderings (orthogonality, residual, swaps sent to
-// the double-double retry) are a little smaller than they were.
+// and a lane of a product warp works on two items at once); the rounding
+// errors of whole reorderings (orthogonality, residual, swaps sent to the
+// double-double retry) are a little smaller than they were.
 // ---------------------------------------------------------------------------
 // Reflector I - f w w^T with w = (w0, a1, 1) that maps a = (a0, a1, 1) onto
 // -sign(a0) |a| e_0: w0 = a0 + sign(a0) |a|, f = 2 / |w|^2 (taken from the
