@@ -142,13 +142,18 @@ __device__ __forceinline__ double oz_combine_any(const unsigned (&a)[7], int er,
 __device__ __forceinline__ bool oz_plain(int er, int ec) {
     return er == 0 || ec == 0 || (unsigned)(er + ec - 1300) <= 1600u;
 }
-// The same for such exponents, in 64-bit integers: T = H 2^24 + L with |H| < 2^46, |L| < 2^40.  A
-// small T is converted as it is; otherwise 7 bits of L are dropped (rounding
-// towards minus infinity) and kept as a sticky bit in bit 0 of a number of at
-// least 55 bits, so that the one rounding of the conversion is that of T.
-// The epilogue is bound by its integer instructions: this takes about 30 of
-// them where the 128-bit form takes about 80.  With the packed digits, a task
-// of 500 panel rows (w = 128) takes 120 us; it took 137 us.
+// The same for such exponents, in 64-bit integers: T = H 2^24 + L with
+// |H| < 2^46, |L| < 2^40.  A small T is converted as it is; otherwise 7 bits
+// of L are dropped (rounding towards minus infinity) and kept as a sticky bit
+// in bit 0 of a number of at least 55 bits, so that the one rounding of the
+// conversion is that of T.  About 30 integer instructions where the 128-bit
+// form takes about 80.  With the packed digits, a task of 500 panel rows
+// (w = 128) takes 120 us; it took 137 us.
+// What bounds the epilogue is not one pipe.  Of its 19.2K cycles a block of 128
+// rows (16 384 outputs), the 64-bit conversions hold the FP64 pipe for 8.2K, the
+// seven conversions to integers the XU pipe for 7.2K, and the integer
+// instructions, at two a cycle, the ALU for up to 7.7K; each warp goes through
+// tensor-memory read, conversions, combination and store in turn.
 __device__ __forceinline__ double oz_combine(const unsigned (&a)[7], int er, int ec) {
     int D[7];
 #pragma unroll

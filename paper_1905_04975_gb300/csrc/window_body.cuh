@@ -181,17 +181,90 @@ __device__ __forceinline__ void apply_refl3(double w0, double w1, double f, doub
     *x1 = fma(-s, w1, *x1);
     *x2 -= s;
 }
-// The elimination kept for the swaps whose FP32-seeded solution does not
-// converge (out of line: it is rare, and the step loop must fit the
-// instruction caches).
-static __device__ __noinline__ bool sylv22_full(const double* __restrict__ Sp, int ja, double* X) {
-    double D[16];
+
+// What follows a 2|2 swap's Sylvester solution X: reflectors, products and
+// tests, with lim for the block that must vanish (dc0..dc3: this lane's column
+// of D, tb: the bit pattern of 10 eps max|D|).
+__device__ __forceinline__ bool swap22_finish(const double (&X)[4], double dc0, double dc1, double dc2,
+                                              double dc3, unsigned long long tb,
+                                              unsigned long long lim, int l, unsigned hmask,
+                                              int hbase, bool strong, double* z, double* dnrc) {
+    const int r = l & 3, c = l >> 2;
+    // reflector 1 on column 0 of [-X; I], (-x00, -x10, 1, 0); reflector 2 on
+    // rows 1..3 of reflector 1 times column 1, (-x01, -x11, 0, 1)
+    const double w1 = -X[1];
+    double w0, f1, u0, f2;
+    refl3(-X[0], w1, &w0, &f1);
+    const double s1 = fma(w0, -X[2], w1 * -X[3]) * f1;
+    const double q1 = fma(-s1, w1, -X[3]), u1 = -s1;  // (q1, u1, 1)
+    refl3(q1, u1, &u0, &f2);
+    // Qs = (I - f1 w w^T)(I - f2 u u^T), w = (w0, w1, 1, 0), u = (0, u0, u1, 1)
+    const double wu = fma(w1, u0, u1);
+    const double wr = sel4(r, w0, w1, 1.0, 0.0), wc = sel4(c, w0, w1, 1.0, 0.0);
+    const double ur = sel4(r, 0.0, u0, u1, 1.0), uc = sel4(c, 0.0, u0, u1, 1.0);
+    const double ar = f1 * wr;
+    double qs = fma(-ar, wc, (r == c) ? 1.0 : 0.0);
+    qs = fma(-(f2 * uc), fma(-ar, wu, ur), qs);
+    // T = Qs^T D: T[r][c] = sum_a Qs[a][r] D[a][c]
+    double T = __shfl_sync(hmask, qs, hbase + 0 + 4 * r) * dc0;
+    T = fma(__shfl_sync(hmask, qs, hbase + 1 + 4 * r), dc1, T);
+    T = fma(__shfl_sync(hmask, qs, hbase + 2 + 4 * r), dc2, T);
+    T = fma(__shfl_sync(hmask, qs, hbase + 3 + 4 * r), dc3, T);
+    // Dt = T Qs: Dt[r][c] = sum_b T[r][b] Qs[b][c]
+    double Dt = 0.0;
+#pragma unroll
+    for (int bb = 0; bb < 4; ++bb)
+        Dt = fma(__shfl_sync(hmask, T, hbase + r + 4 * bb),
+                 __shfl_sync(hmask, qs, hbase + bb + 4 * c), Dt);
+    // weak test on the lower-left 2x2 block
+    const bool low = (r >= 2 && c < 2);
+    bool pass = !__any_sync(hmask, low && abs_bits(Dt) > lim);
+    const double Dt0 = low ? 0.0 : Dt;
+    if (strong && pass) {
+        // P = Qs Dt0: P[r][b] = sum_a Qs[r][a] Dt0[a][b]
+        double P = 0.0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            P = fma(__shfl_sync(hmask, qs, hbase + r + 4 * a),
+                    __shfl_sync(hmask, Dt0, hbase + a + 4 * c), P);
+        // E = P Qs^T - D: E[r][c] = sum_b P[r][b] Qs[c][b] - D[r][c]
+        double E = 0.0;
+#pragma unroll
+        for (int bb = 0; bb < 4; ++bb)
+            E = fma(__shfl_sync(hmask, P, hbase + r + 4 * bb),
+                    __shfl_sync(hmask, qs, hbase + c + 4 * bb), E);
+        E -= sel4(r, dc0, dc1, dc2, dc3);
+        pass = !__any_sync(hmask, abs_bits(E) > tb);
+    }
+    if (pass) {
+        z[0] = w0;
+        z[1] = w1;
+        z[2] = f1;
+        z[3] = u0;
+        z[4] = u1;
+        z[5] = f2;
+        *dnrc = Dt0;
+        return true;
+    }
+    return false;
+}
+
+// The swap by elimination, for the seeded solutions that do not serve (out of
+// line: it is rare, and the step loop must fit the instruction caches).
+static __device__ __noinline__ bool swap22_elim(const double* __restrict__ Sp, int ja, int l,
+                                                unsigned hmask, int hbase, bool strong,
+                                                unsigned long long tb, double* z, double* dnrc) {
+    double D[16], X[4];
 #pragma unroll
     for (int cc = 0; cc < 4; ++cc)
 #pragma unroll
         for (int rr = 0; rr < 4; ++rr)
             D[cc * 4 + rr] = (rr <= cc + 1) ? Sp[poff(ja + cc) + ja + rr] : 0.0;
-    return sylv22_regs(D, X);
+    if (!sylv22_regs(D, X)) return false;
+    const int c = l >> 2;
+    const double* cc = Sp + poff(ja + c) + ja;
+    return swap22_finish(X, cc[0], cc[1], c >= 1 ? cc[2] : 0.0, c >= 2 ? cc[3] : 0.0, tb, tb, l, hmask,
+                         hbase, strong, z, dnrc);
 }
 
 // 2|2 swap by 16 lanes: lane l of the half-warp owns entry (r, c) =
@@ -311,72 +384,8 @@ __device__ __forceinline__ bool swap22_halfwarp(const double* __restrict__ Sp, i
     }
 #pragma unroll
     for (int t = 0; t < 4; ++t) X[t] = __shfl_sync(hmask, own, hbase + t);
-#pragma unroll 1
-    for (;; good = false) {
-        if (!good) {
-            double Xf[4];
-            if (!sylv22_full(Sp, ja, Xf)) return false;
-#pragma unroll
-            for (int t = 0; t < 4; ++t) X[t] = Xf[t];
-        }
-        // reflector 1 on column 0 of [-X; I], (-x00, -x10, 1, 0); reflector 2 on
-        // rows 1..3 of reflector 1 times column 1, (-x01, -x11, 0, 1)
-        const double w1 = -X[1];
-        double w0, f1, u0, f2;
-        refl3(-X[0], w1, &w0, &f1);
-        const double s1 = fma(w0, -X[2], w1 * -X[3]) * f1;
-        const double q1 = fma(-s1, w1, -X[3]), u1 = -s1;  // (q1, u1, 1)
-        refl3(q1, u1, &u0, &f2);
-        // Qs = (I - f1 w w^T)(I - f2 u u^T), w = (w0, w1, 1, 0), u = (0, u0, u1, 1)
-        const double wu = fma(w1, u0, u1);
-        const double wr = sel4(r, w0, w1, 1.0, 0.0), wc = sel4(c, w0, w1, 1.0, 0.0);
-        const double ur = sel4(r, 0.0, u0, u1, 1.0), uc = sel4(c, 0.0, u0, u1, 1.0);
-        const double ar = f1 * wr;
-        double qs = fma(-ar, wc, (r == c) ? 1.0 : 0.0);
-        qs = fma(-(f2 * uc), fma(-ar, wu, ur), qs);
-        // T = Qs^T D: T[r][c] = sum_a Qs[a][r] D[a][c]
-        double T = __shfl_sync(hmask, qs, hbase + 0 + 4 * r) * dc0;
-        T = fma(__shfl_sync(hmask, qs, hbase + 1 + 4 * r), dc1, T);
-        T = fma(__shfl_sync(hmask, qs, hbase + 2 + 4 * r), dc2, T);
-        T = fma(__shfl_sync(hmask, qs, hbase + 3 + 4 * r), dc3, T);
-        // Dt = T Qs: Dt[r][c] = sum_b T[r][b] Qs[b][c]
-        double Dt = 0.0;
-#pragma unroll
-        for (int bb = 0; bb < 4; ++bb)
-            Dt = fma(__shfl_sync(hmask, T, hbase + r + 4 * bb),
-                     __shfl_sync(hmask, qs, hbase + bb + 4 * c), Dt);
-        // weak test on the lower-left 2x2 block
-        const bool low = (r >= 2 && c < 2);
-        bool pass = !__any_sync(hmask, low && abs_bits(Dt) > (good ? tb4 : tb));
-        const double Dt0 = low ? 0.0 : Dt;
-        if (strong && pass) {
-            // P = Qs Dt0: P[r][b] = sum_a Qs[r][a] Dt0[a][b]
-            double P = 0.0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-                P = fma(__shfl_sync(hmask, qs, hbase + r + 4 * a),
-                        __shfl_sync(hmask, Dt0, hbase + a + 4 * c), P);
-            // E = P Qs^T - D: E[r][c] = sum_b P[r][b] Qs[c][b] - D[r][c]
-            double E = 0.0;
-#pragma unroll
-            for (int bb = 0; bb < 4; ++bb)
-                E = fma(__shfl_sync(hmask, P, hbase + r + 4 * bb),
-                        __shfl_sync(hmask, qs, hbase + c + 4 * bb), E);
-            E -= sel4(r, dc0, dc1, dc2, dc3);
-            pass = !__any_sync(hmask, abs_bits(E) > tb);
-        }
-        if (pass) {
-            z[0] = w0;
-            z[1] = w1;
-            z[2] = f1;
-            z[3] = u0;
-            z[4] = u1;
-            z[5] = f2;
-            *dnrc = Dt0;
-            return true;
-        }
-        if (!good) return false;
-    }
+    if (good && swap22_finish(X, dc0, dc1, dc2, dc3, tb, tb4, l, hmask, hbase, strong, z, dnrc)) return true;
+    return swap22_elim(Sp, ja, l, hmask, hbase, strong, tb, z, dnrc);
 }
 
 // k = 3 swap by four lanes (all 32 lanes of the warp call it, eight swaps at a
