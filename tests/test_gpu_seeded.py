@@ -61,7 +61,9 @@ def values(tmp_path_factory):
     r[5000:10000] *= 2.0 ** rng.integers(-60, 61, (5000, 3))
     r[10000:15000, 0] *= 2.0 ** rng.integers(-400, 401, 5000)
     r[10000:15000, 1:] = r[10000:15000, :1] * rng.standard_normal((5000, 2))
-    r[15000:] = np.round(3 * r[15000:])
+    r[15000:18000] = np.round(3 * r[15000:18000])
+    r[18000:19000, 1] *= 1e-9  # almost no rotation
+    r[19000:, 0] *= 1e-9       # almost an exchange
     x = np.concatenate([np.array(ex), r])
     x[:, 1] = np.where((x[:, 0] == 0) & (x[:, 1] == 0) & (x[:, 2] == 0), 1.0, x[:, 1])
     n = x.shape[0]
@@ -90,6 +92,17 @@ def test_rotation(values):
     n = np.hypot(x[k], y[k])
     c, s = o[2][k].astype(LD), o[3][k].astype(LD)
     assert np.max(np.abs(c - x[k] / n)) <= 5 * U and np.max(np.abs(s - y[k] / n)) <= 5 * U
+
+
+def test_rotation_by_almost_nothing(values):
+    """Many such rotations are accumulated: their rounding errors must not have
+    a mean.  The larger component is its correctly rounded value, 1; the other's
+    square does not count."""
+    (x, y, _), o = values
+    for a, b in ((0, 1), (1, 0)):
+        p = (x, y)
+        k = np.abs(p[b]) * 2.0 ** 29 < np.abs(p[a])
+        assert k.sum() > 500 and np.all(np.abs(o[2 + a][k]) == 1.0)
 
 
 def test_reflector(values):
